@@ -11,6 +11,17 @@ using rsdev::FieldDev;
 using rsdev::ShootDesc;
 using namespace rshost;
 
+namespace {
+
+// Offset of the float-float partials (float4 per listed ray) behind the re-evaluation list {16-byte
+// header, cap entries of 8 bytes} at list_off: rounded up to the 16 bytes a float4 access needs, as an
+// odd capacity (rays / 32 of the call) ends the list half way.
+size_t staged_ff_offset(size_t list_off, unsigned cap) {
+  return list_off + (16 + sizeof(uint2) * (size_t)cap + 15) / 16 * 16;
+}
+
+}  // namespace
+
 extern "C" {
 
 int rs_set_staged_state_budget(uint64_t bytes) {
@@ -52,7 +63,7 @@ int rs_shoot_staged(int n_parts, const rs_field_t* parts, const rs_ray_grid* g, 
   const size_t state_bytes = rsint::staged_state_bytes(rows_max, d.n0);
   const unsigned cap = g_certify ? rsint::recheck_capacity(rows_max * d.n0) : 0u;
   const size_t list_off = (state_bytes + 255) / 256 * 256;
-  const size_t ff_off = list_off + 16 + sizeof(uint2) * (size_t)cap;
+  const size_t ff_off = staged_ff_offset(list_off, cap);
   void* ws = nullptr;
   cudaError_t e = dev_alloc_async(&ws, ff_off + sizeof(float4) * (size_t)cap, s);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (staged-shoot workspace)");
@@ -173,7 +184,7 @@ int rs_shoot_streamed(const float* h_lens_xy, const float* h_masses, int64_t n_l
   const size_t state_bytes = rsint::staged_state_bytes(rows_max, d.n0);
   const unsigned cap = g_certify ? rsint::recheck_capacity(rows_max * d.n0) : 0u;
   const size_t list_off = (state_bytes + 255) / 256 * 256;
-  const size_t ff_off = list_off + 16 + sizeof(uint2) * (size_t)cap;
+  const size_t ff_off = staged_ff_offset(list_off, cap);
   if (e == cudaSuccess) e = dev_alloc(&r.ws, ff_off + sizeof(float4) * (size_t)cap);
   if (e != cudaSuccess) return cuda_fail(e, "streamed-shoot resources");
   char* base = reinterpret_cast<char*>(r.ws);

@@ -63,6 +63,21 @@ def test_row_blocks_and_rows_match():
     assert np.array_equal(got_rows, ref_rows) and o_rows == oref_rows
 
 
+@pytest.mark.parametrize("side", [363, 37])
+def test_odd_list_capacity(side):
+    """rays / 32 odd (4117, and 1369 below the minimum): the float-float partials behind a list of odd capacity
+    still start on 16 bytes, resident and streamed."""
+    m = rs()
+    spec = ri.disc_field("sto", 1100, 0.5, 0.1, 0.25, side, 48, seed=6, mass="salpeter")
+    ref, oref = shoot_gpu(spec)
+    got, o = _staged(spec, [512])
+    assert np.array_equal(got, ref) and o == oref
+    c = torch.zeros((48, 48), dtype=torch.int32, device=dev())
+    o = torch.zeros(1, dtype=torch.int64, device=dev())
+    m.rs_shoot_streamed(spec.lens_xy, spec.masses, spec.kappa_c, spec.gamma, 1024, spec.grid, 0, side, spec.window, c, o)
+    assert np.array_equal(c.cpu().numpy().view(np.uint32), ref) and int(o.item()) == oref
+
+
 def test_partition_validation():
     m = rs()
     spec = ri.disc_field("stv", 600, 0.4, 0.0, 0.3, 256, 32, seed=2, mass="equal")
