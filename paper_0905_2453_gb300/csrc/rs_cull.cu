@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(128, 2) shoot_cells_kernel(const ShootDesc d, 
     float a1h[RPT], a1l[RPT], a2h[RPT], a2l[RPT], sig[RPT], tn[RPT];
     if (!deflect_pairs<RPT, rsint::kTile, MASS, false, 1>(d.f, x1, x2, a1h, a1l, a2h, a2l, sig, tn, sm, ps, &ns))
       return;
-    bin_rays<RPT, 1>(d, x1, x2, a1h, a1l, a2h, a2l, sig, tn, valid, jrel, i_base, lane);
+    bin_rays<RPT, RPT, 1>(d, x1, x2, a1h, a1l, a2h, a2l, sig, tn, valid, jrel, i_base, lane);
   }
 }
 

@@ -1,7 +1,7 @@
 // Device side of the inverse ray-shooting path (sm_103a).
 //
 // What one CTA computes: a tile of BLOCK x RPT rays of a regular image-plane
-// grid (one grid row per warp), deflected by all lenses of a field (Eq. 2, a
+// grid (two grid rows per warp), deflected by all lenses of a field (Eq. 2, a
 // direct sum; the paper's ray x lens decomposition of Eq. 5 with lens tiles
 // staged through shared memory, Section 2.2), mapped to the source plane with
 // the macro-model of Eq. 6 and binned into a uint32 count map (Eq. 4 counts).
@@ -13,9 +13,10 @@
 //   * Lenses are stored duplicated, {x1, x1, x2, x2} (and {m, m}), so one
 //     shared-memory load yields the 64-bit operand pairs of the packed
 //     f32x2 instructions: every packed op advances two rays against one lens.
-//   * The rays of a warp share one grid row, so (x2 - x2_lens) and its square
-//     come from a per-row table built in shared memory once per lens tile.
-//   * Per lens and ray pair: sub.f32x2, fma.f32x2 (|d|^2), the reciprocal,
+//   * The rays of a thread are two grid rows by two column pairs: (x2 - x2_lens)
+//     and its square come from a per-row table built in shared memory once per
+//     lens tile, and (x1 - x1_lens) of a column pair serves both its rows.
+//   * Per lens and ray pair: half a sub.f32x2, fma.f32x2 (|d|^2), the reciprocal,
 //     [mul.f32x2 by the mass], fma.f32x2 x2 -- the ten flops per interaction of
 //     the paper's Appendix A.  For three of every four lens pairs (unit masses;
 //     one of two with masses) one rcp.approx of the product of the two squared
@@ -359,6 +360,7 @@ struct __align__(16) LensSmem {
   float4 lens4[2][TILE];     // double-buffered lens tiles {x1, x1, x2, x2}
   float2 mass2[2][TILE];     // {m, m}
   float4 rowtab[ROWS][TILE]; // per CTA row r and lens l of the current tile: {d2, d2, d2^2, d2^2}
+  float2 x1tab[ROWS > 1 ? TILE : 2];  // {x1, x1} of the current tile's lenses: a lens pair in one 16-byte load
   float x2row[ROWS];         // x2 of the CTA's rows
   float x1col[kMaxSeg];      // x1 of the CTA's columns (shoot_tile)
   uint64_t bar[2];
@@ -404,7 +406,7 @@ __device__ __forceinline__ float ray_coord(int64_t idx, double spacing, double o
 
 // ----------------------------------------------------------------------------------------------
 // Lens-pair step.  Two consecutive lenses a, b against one ray pair (lanes A, B of each operand).
-// d1 = x1 - x1_lens; r2 = d1^2 + d2^2 with d2^2 (S2) supplied; w = m / r2; P += w * (d1, d2).
+// With d1 = x1 - x1_lens, d2 and d2^2 (S2) supplied: r2 = d1^2 + d2^2; w = m / r2; P += w * (d1, d2).
 //
 // MONT: one reciprocal serves both lenses (Montgomery's simultaneous inversion):
 //   inv = 1 / (r2a * r2b),  1/r2a = r2b * inv,  1/r2b = r2a * inv.
@@ -414,11 +416,8 @@ __device__ __forceinline__ float ray_coord(int64_t idx, double spacing, double o
 // deflection is then ~1e9 (out of any window), and only that ray is affected.
 // ----------------------------------------------------------------------------------------------
 template <bool MONT, bool MASS>
-__device__ __forceinline__ void lens_pair_step(uint64_t X1, uint64_t Lxa, uint64_t Lxb, uint64_t D2a, uint64_t S2a,
-                                               uint64_t D2b, uint64_t S2b, uint64_t Ma, uint64_t Mb, uint64_t& P1,
-                                               uint64_t& P2) {
-  const uint64_t d1a = f2_sub(X1, Lxa);
-  const uint64_t d1b = f2_sub(X1, Lxb);
+__device__ __forceinline__ void lens_pair_step(uint64_t d1a, uint64_t d1b, uint64_t D2a, uint64_t S2a, uint64_t D2b,
+                                               uint64_t S2b, uint64_t Ma, uint64_t Mb, uint64_t& P1, uint64_t& P2) {
   const uint64_t r2a = f2_fma(d1a, d1a, S2a);
   const uint64_t r2b = f2_fma(d1b, d1b, S2b);
   uint64_t wa, wb;
@@ -448,9 +447,8 @@ __device__ __forceinline__ void lens_pair_step(uint64_t X1, uint64_t Lxa, uint64
 
 // A single lens (the odd last lens of a field), direct reciprocal.
 template <bool MASS>
-__device__ __forceinline__ void lens_single_step(uint64_t X1, uint64_t Lx, uint64_t D2, uint64_t S2, uint64_t M,
-                                                 uint64_t& P1, uint64_t& P2) {
-  const uint64_t d1 = f2_sub(X1, Lx);
+__device__ __forceinline__ void lens_single_step(uint64_t d1, uint64_t D2, uint64_t S2, uint64_t M, uint64_t& P1,
+                                                 uint64_t& P2) {
   const uint64_t r2 = f2_fma(d1, d1, S2);
   float a0, a1;
   f2_unpack(r2, a0, a1);
@@ -477,33 +475,121 @@ __device__ __forceinline__ void load_lens(uint32_t lbase, uint32_t mbase, int l,
   M = MASS ? lds_pair(mbase + (uint32_t)l * 8u) : 0ull;
 }
 
-// One lens pair (lenses l, l + 1) against all ray pairs of the thread.
-// ROW: all rays of the thread share x2 (one grid row); d2 and d2^2 of the row come from the
-// shared-memory row table built once per lens tile (rt = that row's table).  Otherwise each ray
-// pair forms them itself.  Either way every ray gets exactly the same operations.
-template <int NP, bool MONT, bool MASS, bool ROW>
-__device__ __forceinline__ void lens_pair_all(uint32_t lbase, uint32_t mbase, uint32_t rt, int l,
-                                              const uint64_t (&X1)[NP], const uint64_t (&X2)[NP], uint64_t (&P1)[NP],
-                                              uint64_t (&P2)[NP]) {
+// One lens pair (lenses l, l + 1) against all ray pairs of the thread, every ray pair with its own
+// x2 (listed rays, cells): d2 and d2^2 are formed per ray pair.
+template <int NP, bool MONT, bool MASS>
+__device__ __forceinline__ void lens_pair_all(uint32_t lbase, uint32_t mbase, int l, const uint64_t (&X1)[NP],
+                                              const uint64_t (&X2)[NP], uint64_t (&P1)[NP], uint64_t (&P2)[NP]) {
   uint64_t Lxa, Lya, Ma, Lxb, Lyb, Mb;
-  if (ROW) {
-    Lxa = lds_pair(lbase + (uint32_t)l * 16u);
-    Lxb = lds_pair(lbase + (uint32_t)(l + 1) * 16u);
-    Ma = MASS ? lds_pair(mbase + (uint32_t)l * 8u) : 0ull;
-    Mb = MASS ? lds_pair(mbase + (uint32_t)(l + 1) * 8u) : 0ull;
-    uint64_t D2a, S2a, D2b, S2b;
-    lds_pair2(rt + (uint32_t)l * 16u, D2a, S2a);
-    lds_pair2(rt + (uint32_t)(l + 1) * 16u, D2b, S2b);
+  load_lens<MASS>(lbase, mbase, l, Lxa, Lya, Ma);
+  load_lens<MASS>(lbase, mbase, l + 1, Lxb, Lyb, Mb);
 #pragma unroll
-    for (int q = 0; q < NP; ++q) lens_pair_step<MONT, MASS>(X1[q], Lxa, Lxb, D2a, S2a, D2b, S2b, Ma, Mb, P1[q], P2[q]);
-  } else {
-    load_lens<MASS>(lbase, mbase, l, Lxa, Lya, Ma);
-    load_lens<MASS>(lbase, mbase, l + 1, Lxb, Lyb, Mb);
+  for (int q = 0; q < NP; ++q) {
+    const uint64_t D2a = f2_sub(X2[q], Lya), D2b = f2_sub(X2[q], Lyb);
+    const uint64_t S2a = f2_mul(D2a, D2a), S2b = f2_mul(D2b, D2b);
+    lens_pair_step<MONT, MASS>(f2_sub(X1[q], Lxa), f2_sub(X1[q], Lxb), D2a, S2a, D2b, S2b, Ma, Mb, P1[q], P2[q]);
+  }
+}
+
+// The same for a thread whose rays form a tile of R grid rows by CP column pairs (ray pair q = r CP + c):
+// d2 and d2^2 of each row come from the shared-memory row table built once per lens tile (rt: the
+// thread's first row, rows TILE entries apart), and d1 = x1 - x1_lens of a column pair is formed once
+// for its R rows.  Every ray gets exactly the operations of lens_pair_all.
+//
+// The kernel is bound by the FMA pipe together with the register reads that feed it (a packed FMA of
+// three distinct operands takes three cycles of a sub-core, not two), so an operation shared between rows
+// is worth its full issue time: two rows take 4.625 packed operations per ray pair and lens instead of
+// 5.125.  Body alone, 1e4 unit-mass lenses, 4096^2 rays: one row of eight columns 29.6 ms, two rows of
+// four 27.7 ms; four rows of four (16 rays per thread) 27.4 ms but with half the warps to cover a CTA's
+// start and end, so two rows are kept.
+template <int R, int CP, int TILE, bool MONT, bool MASS>
+__device__ __forceinline__ void lens_pair_rows(uint32_t xbase, uint32_t mbase, uint32_t rt, int l,
+                                               const uint64_t (&X1)[R * CP], uint64_t (&P1)[R * CP],
+                                               uint64_t (&P2)[R * CP]) {
+  uint64_t Lxa, Lxb, Ma = 0ull, Mb = 0ull, D2a[R], S2a[R], D2b[R], S2b[R];
+  lds_pair2(xbase + (uint32_t)l * 8u, Lxa, Lxb);  // l is even: 16-byte aligned
+  if (MASS) lds_pair2(mbase + (uint32_t)l * 8u, Ma, Mb);
 #pragma unroll
-    for (int q = 0; q < NP; ++q) {
-      const uint64_t D2a = f2_sub(X2[q], Lya), D2b = f2_sub(X2[q], Lyb);
-      const uint64_t S2a = f2_mul(D2a, D2a), S2b = f2_mul(D2b, D2b);
-      lens_pair_step<MONT, MASS>(X1[q], Lxa, Lxb, D2a, S2a, D2b, S2b, Ma, Mb, P1[q], P2[q]);
+  for (int r = 0; r < R; ++r) {
+    lds_pair2(rt + (uint32_t)(r * TILE + l) * 16u, D2a[r], S2a[r]);
+    lds_pair2(rt + (uint32_t)(r * TILE + l + 1) * 16u, D2b[r], S2b[r]);
+  }
+#pragma unroll
+  for (int c = 0; c < CP; ++c) {
+    const uint64_t d1a = f2_sub(X1[c], Lxa), d1b = f2_sub(X1[c], Lxb);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      lens_pair_step<MONT, MASS>(d1a, d1b, D2a[r], S2a[r], D2b[r], S2b[r], Ma, Mb, P1[r * CP + c], P2[r * CP + c]);
+  }
+}
+
+// A thread's RPT rays on a shoot tile: R grid rows by CP column pairs, a warp 32 x 2 CP columns of those
+// rows, and the CTA's warps side by side in WC columns of warps -- W rows by 32 RPT columns per CTA of W
+// warps whatever R is (six rays per thread do not split into two rows of pairs).
+template <int RPT>
+struct RayTile {
+  static constexpr int R = RPT % 4 == 0 ? 2 : 1;
+  static constexpr int CP = RPT / (2 * R);
+  static constexpr int WC = R;
+};
+
+template <int RPT, int TILE, bool MONT, bool MASS, bool ROW>
+__device__ __forceinline__ void lens_pair_any(uint32_t lbase, uint32_t xbase, uint32_t mbase, uint32_t rt, int l,
+                                              const uint64_t (&X1)[RPT / 2], const uint64_t (&X2)[RPT / 2],
+                                              uint64_t (&P1)[RPT / 2], uint64_t (&P2)[RPT / 2]) {
+  if constexpr (ROW)
+    lens_pair_rows<RayTile<RPT>::R, RayTile<RPT>::CP, TILE, MONT, MASS>(xbase, mbase, rt, l, X1, P1, P2);
+  else
+    lens_pair_all<RPT / 2, MONT, MASS>(lbase, mbase, l, X1, X2, P1, P2);
+}
+
+// Four lens pairs of a group (lenses l .. l + 7, l a multiple of 8 within the group): the fixed reciprocal pattern.
+template <int RPT, int TILE, bool MASS, bool ROW>
+__device__ __forceinline__ void lens_block(uint32_t lbase, uint32_t xbase, uint32_t mbase, uint32_t rt, int l,
+                                           const uint64_t (&X1)[RPT / 2], const uint64_t (&X2)[RPT / 2],
+                                           uint64_t (&P1)[RPT / 2], uint64_t (&P2)[RPT / 2]) {
+  lens_pair_any<RPT, TILE, mont_pair<MASS>(0), MASS, ROW>(lbase, xbase, mbase, rt, l + 0, X1, X2, P1, P2);
+  lens_pair_any<RPT, TILE, mont_pair<MASS>(1), MASS, ROW>(lbase, xbase, mbase, rt, l + 2, X1, X2, P1, P2);
+  lens_pair_any<RPT, TILE, mont_pair<MASS>(2), MASS, ROW>(lbase, xbase, mbase, rt, l + 4, X1, X2, P1, P2);
+  lens_pair_any<RPT, TILE, mont_pair<MASS>(3), MASS, ROW>(lbase, xbase, mbase, rt, l + 6, X1, X2, P1, P2);
+}
+
+// The last, partial group of a field (cnt < 64 lenses from l0): the same pattern by pair index, an odd last
+// lens directly.
+template <int RPT, int TILE, bool MASS, bool ROW>
+__device__ __forceinline__ void lens_group_partial(uint32_t lbase, uint32_t xbase, uint32_t mbase, uint32_t rt, int l0,
+                                                   int cnt, const uint64_t (&X1)[RPT / 2],
+                                                   const uint64_t (&X2)[RPT / 2], uint64_t (&P1)[RPT / 2],
+                                                   uint64_t (&P2)[RPT / 2]) {
+  int p = 0;
+  for (; 2 * p + 8 <= cnt; p += 4)  // whole blocks of four pairs first (p = 0 mod 4 at each)
+    lens_block<RPT, TILE, MASS, ROW>(lbase, xbase, mbase, rt, l0 + 2 * p, X1, X2, P1, P2);
+  for (; 2 * p + 1 < cnt; ++p) {
+    if (mont_pair<MASS>(p))
+      lens_pair_any<RPT, TILE, true, MASS, ROW>(lbase, xbase, mbase, rt, l0 + 2 * p, X1, X2, P1, P2);
+    else
+      lens_pair_any<RPT, TILE, false, MASS, ROW>(lbase, xbase, mbase, rt, l0 + 2 * p, X1, X2, P1, P2);
+  }
+  if (2 * p < cnt) {
+    const int l = l0 + 2 * p;
+    uint64_t Lx, Ly, M;
+    load_lens<MASS>(lbase, mbase, l, Lx, Ly, M);
+    if constexpr (ROW) {
+      constexpr int R = RayTile<RPT>::R, CP = RayTile<RPT>::CP;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        uint64_t D2, S2;
+        lds_pair2(rt + (uint32_t)(r * TILE + l) * 16u, D2, S2);
+#pragma unroll
+        for (int c = 0; c < CP; ++c)
+          lens_single_step<MASS>(f2_sub(X1[c], Lx), D2, S2, M, P1[r * CP + c], P2[r * CP + c]);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < RPT / 2; ++q) {
+        const uint64_t D2 = f2_sub(X2[q], Ly);
+        lens_single_step<MASS>(f2_sub(X1[q], Lx), D2, f2_mul(D2, D2), M, P1[q], P2[q]);
+      }
     }
   }
 }
@@ -515,7 +601,9 @@ template <int TILE, int ROWS>
 __device__ __forceinline__ void build_row_table(LensSmem<TILE, ROWS>& sm, int b, int cnt) {
   constexpr int BLOCK = ROWS * 32;
   for (int l = threadIdx.x; l < cnt; l += BLOCK) {
-    const float y = sm.lens4[b][l].z;
+    const float4 L = sm.lens4[b][l];
+    const float y = L.z;
+    sm.x1tab[l] = make_float2(L.x, L.x);
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
       const uint64_t D2 = f2_sub(f2_pack(sm.x2row[r], sm.x2row[r]), f2_pack(y, y));
@@ -530,8 +618,8 @@ __device__ __forceinline__ void build_row_table(LensSmem<TILE, ROWS>& sm, int b,
 
 // ----------------------------------------------------------------------------------------------
 // Deflection of RPT rays per thread by all lenses of the field (Eq. 2).
-// x1/x2: ray coordinates (ROW: all rays of a warp share x2, recorded in sm.x2row[warp] by the
-// caller).  alpha1/alpha2 (double) out.  Returns false if a bounded wait gave up (the CTA must
+// x1/x2: ray coordinates (ROW: the thread's rays are R rows by CP column pairs as RayTile lays them out,
+// the x2 of the CTA's rows recorded in sm.x2row by the caller).  alpha1/alpha2 (double) out.  Returns false if a bounded wait gave up (the CTA must
 // then stop; the status word has been set).  The arithmetic per ray depends only on the ray and
 // the field.
 // ----------------------------------------------------------------------------------------------
@@ -542,29 +630,40 @@ struct DeflectAcc {
   uint64_t H1[NP], L1[NP], H2[NP], L2[NP], SS[NP], AB[NP];
 };
 
+// Folds a group's partial sums into the accumulators.
+template <int NP>
+__device__ __forceinline__ void fold_group(DeflectAcc<NP>& a, const uint64_t (&P1)[NP], const uint64_t (&P2)[NP]) {
+#pragma unroll
+  for (int q = 0; q < NP; ++q) {
+    twosum_accumulate(a.H1[q], a.L1[q], P1[q]);
+    twosum_accumulate(a.H2[q], a.L2[q], P2[q]);
+    a.SS[q] = f2_fma(P1[q], P1[q], a.SS[q]);
+    a.SS[q] = f2_fma(P2[q], P2[q], a.SS[q]);
+    a.AB[q] = f2_add_x(a.AB[q], f2_add_x(f2_abs(P1[q]), f2_abs(P2[q])));
+  }
+}
+
 // Accumulate the field's lenses into acc (X1/X2: packed ray coordinates).  The arithmetic depends on
 // a lens's index within the field only through the group (64) and renormalisation (256) schedule,
 // so a field split into parts of multiples of 256 lenses, accumulated part after part, gives
 // bitwise the sums of the whole field.  Returns false if a bounded wait gave up (the CTA must then
 // stop; the status word has been set).
 // With a near-lens search (NS::kOn), every tile's lenses inside the group boxes of ns are listed and
-// their near terms folded into ns.t (the caller sets the boxes and the thread's ns.t entries).
+// their near terms folded into ns.t (the caller sets the boxes and the thread's ns.t entries).  A warp
+// without a ray of the call (active false, warp-uniform) takes part in the copies, tables and barriers only.
 template <int RPT, int TILE, bool MASS, bool ROW, int ROWS, class NS = NoNear>
 __device__ __forceinline__ bool deflect_accumulate(const FieldDev& f, const uint64_t (&X1)[RPT / 2],
                                                    const uint64_t (&X2)[RPT / 2], DeflectAcc<RPT / 2>& acc,
-                                                   LensSmem<TILE, ROWS>& sm, PipeState& ps, NS* ns = nullptr) {
+                                                   LensSmem<TILE, ROWS>& sm, PipeState& ps, NS* ns = nullptr,
+                                                   bool active = true) {
   static_assert(TILE % kGroup == 0 && kGroup % 8 == 0, "lens tile must hold whole lens groups");
   static_assert(kRenorm % kGroup == 0, "renormalisation falls on group boundaries");
   constexpr int NP = RPT / 2;
-  uint64_t (&H1)[NP] = acc.H1;
-  uint64_t (&L1)[NP] = acc.L1;
-  uint64_t (&H2)[NP] = acc.H2;
-  uint64_t (&L2)[NP] = acc.L2;
-  uint64_t (&SS)[NP] = acc.SS;
-  uint64_t (&AB)[NP] = acc.AB;
   const int n = f.n_lens;
   const int ntiles = (n + TILE - 1) / TILE;
-  const uint32_t rt = smem_u32(&sm.rowtab[ROW ? (threadIdx.x >> 5) : 0][0]);
+  // the thread's first row of the CTA (shoot tiles: RayTile)
+  const uint32_t rt = smem_u32(
+      &sm.rowtab[ROW ? (int)(threadIdx.x >> 5) / RayTile<RPT>::WC * RayTile<RPT>::R : 0][0]);
   bool ok = true;
   if (threadIdx.x == 0) {
     if (ntiles > 0) issue_lens_tile<TILE, MASS>(f, sm, 0, 0);
@@ -591,77 +690,32 @@ __device__ __forceinline__ bool deflect_accumulate(const FieldDev& f, const uint
       near_gather<TILE>(*ns, t & 1, &sm.lens4[b][0], cnt, t * TILE, (int)(blockDim.x >> 5));
     }
     const uint32_t lbase = smem_u32(&sm.lens4[b][0]);
+    const uint32_t xbase = smem_u32(&sm.x1tab[0]);
     const uint32_t mbase = smem_u32(&sm.mass2[b][0]);
-    int g = 0;
-    for (; g + kGroup <= cnt; g += kGroup) {
-      uint64_t P1[NP], P2[NP];
+    if (active) {
+      int g = 0;
+      for (; g + kGroup <= cnt; g += kGroup) {
+        uint64_t P1[NP], P2[NP];
 #pragma unroll
-      for (int q = 0; q < NP; ++q) P1[q] = P2[q] = 0ull;
+        for (int q = 0; q < NP; ++q) P1[q] = P2[q] = 0ull;
 #pragma unroll
-      for (int p4 = 0; p4 < kGroup / 8; ++p4) {  // blocks of four lens pairs: fixed reciprocal pattern
-        const int l = g + p4 * 8;
-        lens_pair_all<NP, mont_pair<MASS>(0), MASS, ROW>(lbase, mbase, rt, l + 0, X1, X2, P1, P2);
-        lens_pair_all<NP, mont_pair<MASS>(1), MASS, ROW>(lbase, mbase, rt, l + 2, X1, X2, P1, P2);
-        lens_pair_all<NP, mont_pair<MASS>(2), MASS, ROW>(lbase, mbase, rt, l + 4, X1, X2, P1, P2);
-        lens_pair_all<NP, mont_pair<MASS>(3), MASS, ROW>(lbase, mbase, rt, l + 6, X1, X2, P1, P2);
-      }
-#pragma unroll
-      for (int q = 0; q < NP; ++q) {
-        twosum_accumulate(H1[q], L1[q], P1[q]);
-        twosum_accumulate(H2[q], L2[q], P2[q]);
-        SS[q] = f2_fma(P1[q], P1[q], SS[q]);
-        SS[q] = f2_fma(P2[q], P2[q], SS[q]);
-        AB[q] = f2_add_x(AB[q], f2_add_x(f2_abs(P1[q]), f2_abs(P2[q])));
-      }
-      if ((t * TILE + g + kGroup) % kRenorm == 0) {  // CTA-uniform
-#pragma unroll
-        for (int q = 0; q < NP; ++q) {
-          renormalise(H1[q], L1[q]);
-          renormalise(H2[q], L2[q]);
-        }
-      }
-    }
-    if (g < cnt) {  // last, partial group of the field: same pattern by pair index, odd lens direct
-      uint64_t P1[NP], P2[NP];
-#pragma unroll
-      for (int q = 0; q < NP; ++q) P1[q] = P2[q] = 0ull;
-      int p = 0;
-      for (; g + 2 * p + 8 <= cnt; p += 4) {  // whole blocks of four pairs first (p = 0 mod 4 at each)
-        lens_pair_all<NP, mont_pair<MASS>(0), MASS, ROW>(lbase, mbase, rt, g + 2 * p + 0, X1, X2, P1, P2);
-        lens_pair_all<NP, mont_pair<MASS>(1), MASS, ROW>(lbase, mbase, rt, g + 2 * p + 2, X1, X2, P1, P2);
-        lens_pair_all<NP, mont_pair<MASS>(2), MASS, ROW>(lbase, mbase, rt, g + 2 * p + 4, X1, X2, P1, P2);
-        lens_pair_all<NP, mont_pair<MASS>(3), MASS, ROW>(lbase, mbase, rt, g + 2 * p + 6, X1, X2, P1, P2);
-      }
-      for (; g + 2 * p + 1 < cnt; ++p) {
-        if (mont_pair<MASS>(p))
-          lens_pair_all<NP, true, MASS, ROW>(lbase, mbase, rt, g + 2 * p, X1, X2, P1, P2);
-        else
-          lens_pair_all<NP, false, MASS, ROW>(lbase, mbase, rt, g + 2 * p, X1, X2, P1, P2);
-      }
-      if (g + 2 * p < cnt) {
-        const int l = g + 2 * p;
-        uint64_t Lx, Ly, M;
-        load_lens<MASS>(lbase, mbase, l, Lx, Ly, M);
-        if (ROW) {
-          uint64_t D2, S2;
-          lds_pair2(rt + (uint32_t)l * 16u, D2, S2);
-#pragma unroll
-          for (int q = 0; q < NP; ++q) lens_single_step<MASS>(X1[q], Lx, D2, S2, M, P1[q], P2[q]);
-        } else {
+        for (int p4 = 0; p4 < kGroup / 8; ++p4)
+          lens_block<RPT, TILE, MASS, ROW>(lbase, xbase, mbase, rt, g + p4 * 8, X1, X2, P1, P2);
+        fold_group<NP>(acc, P1, P2);
+        if ((t * TILE + g + kGroup) % kRenorm == 0) {  // CTA-uniform
 #pragma unroll
           for (int q = 0; q < NP; ++q) {
-            const uint64_t D2 = f2_sub(X2[q], Ly);
-            lens_single_step<MASS>(X1[q], Lx, D2, f2_mul(D2, D2), M, P1[q], P2[q]);
+            renormalise(acc.H1[q], acc.L1[q]);
+            renormalise(acc.H2[q], acc.L2[q]);
           }
         }
       }
+      if (g < cnt) {  // last, partial group of the field
+        uint64_t P1[NP], P2[NP];
 #pragma unroll
-      for (int q = 0; q < NP; ++q) {
-        twosum_accumulate(H1[q], L1[q], P1[q]);
-        twosum_accumulate(H2[q], L2[q], P2[q]);
-        SS[q] = f2_fma(P1[q], P1[q], SS[q]);
-        SS[q] = f2_fma(P2[q], P2[q], SS[q]);
-        AB[q] = f2_add_x(AB[q], f2_add_x(f2_abs(P1[q]), f2_abs(P2[q])));
+        for (int q = 0; q < NP; ++q) P1[q] = P2[q] = 0ull;
+        lens_group_partial<RPT, TILE, MASS, ROW>(lbase, xbase, mbase, rt, g, cnt - g, X1, X2, P1, P2);
+        fold_group<NP>(acc, P1, P2);
       }
     }
     __syncthreads();  // every thread is done with buffer b, the row table and the previous tile's near list
@@ -725,7 +779,8 @@ template <int RPT, int TILE, bool MASS, bool ROW, int ROWS, class NS = NoNear>
 __device__ __forceinline__ bool deflect_pairs(const FieldDev& f, const float (&x1)[RPT], const float (&x2)[RPT],
                                               float (&a1h)[RPT], float (&a1l)[RPT], float (&a2h)[RPT],
                                               float (&a2l)[RPT], float (&sig)[RPT], float (&tn)[RPT],
-                                              LensSmem<TILE, ROWS>& sm, PipeState& ps, NS* ns = nullptr) {
+                                              LensSmem<TILE, ROWS>& sm, PipeState& ps, NS* ns = nullptr,
+                                              bool active = true) {
   static_assert(RPT % 2 == 0, "rays per thread must be even (packed pairs)");
   constexpr int NP = RPT / 2;
   uint64_t X1[NP], X2[NP];
@@ -737,7 +792,7 @@ __device__ __forceinline__ bool deflect_pairs(const FieldDev& f, const float (&x
 #pragma unroll
     for (int k = 0; k < RPT; ++k) ns->t[k * blockDim.x + threadIdx.x] = 0.f;
   }
-  if (!deflect_accumulate<RPT, TILE, MASS, ROW, ROWS, NS>(f, X1, X2, acc, sm, ps, ns)) return false;
+  if (!deflect_accumulate<RPT, TILE, MASS, ROW, ROWS, NS>(f, X1, X2, acc, sm, ps, ns, active)) return false;
   deflect_finish<RPT>(acc, a1h, a1l, a2h, a2l, sig);
 #pragma unroll
   for (int k = 0; k < RPT; ++k) {
@@ -840,8 +895,8 @@ __device__ __forceinline__ bool axis_outside(int p, float f, float m, int np) {
 }
 
 // ----------------------------------------------------------------------------------------------
-// Eq. 6 and binning of a thread's RPT rays (ray k at grid column i_base + STRIDE k of call row
-// jrel): counts, the out-of-window count, and, with certified binning, the list of rays to
+// Eq. 6 and binning of a thread's RPT rays (PER consecutive rays per grid row: ray k at grid column
+// i_base + STRIDE (k mod PER) of call row jrel + k / PER): counts, the out-of-window count, and, with certified binning, the list of rays to
 // re-evaluate in float-float.  Every lane of the warp must call it (warp-aggregated atomics).
 //
 // With certified binning most rays are decided from a float32 evaluation of u with a bound on its
@@ -849,7 +904,7 @@ __device__ __forceinline__ bool axis_outside(int p, float f, float m, int np) {
 // outside the window.  The others take the float-float evaluation (ff_pixel) and its narrower margin,
 // and those still uncertain are listed for the float-float re-evaluation over the lenses.
 // ----------------------------------------------------------------------------------------------
-template <int RPT, int STRIDE>
+template <int RPT, int PER, int STRIDE>
 __device__ __forceinline__ void bin_rays(const ShootDesc& d, const float (&x1)[RPT], const float (&x2)[RPT],
                                          const float (&a1h)[RPT], const float (&a1l)[RPT], const float (&a2h)[RPT],
                                          const float (&a2l)[RPT], const float (&sig)[RPT], const float (&tn)[RPT],
@@ -912,8 +967,8 @@ __device__ __forceinline__ void bin_rays(const ShootDesc& d, const float (&x1)[R
         if (need) {
           const unsigned slot = base + (unsigned)__popc(mask & ((1u << lane) - 1u));
           if (slot < d.rc_cap) {
-            const int64_t i = i_base + STRIDE * k;
-            d.rc_list[slot] = make_uint2((unsigned)d.field_id, (unsigned)(jrel * d.n0 + i));
+            const int64_t i = i_base + STRIDE * (k % PER);
+            d.rc_list[slot] = make_uint2((unsigned)d.field_id, (unsigned)((jrel + k / PER) * d.n0 + i));
             bin_now = false;  // counted by the float-float re-evaluation
           } else {
             atomicOr(d.f.status, kStatusListFull);  // list full: the ray keeps its float32 decision
@@ -929,8 +984,9 @@ __device__ __forceinline__ void bin_rays(const ShootDesc& d, const float (&x1)[R
 }
 
 // ----------------------------------------------------------------------------------------------
-// Ray tiles of a shoot call.  A CTA of WARPS warps covers WARPS consecutive grid rows (one per
-// warp) by 32 * RPT consecutive columns; lane l of a warp holds columns c0 + l + 32 k, k < RPT.
+// Ray tiles of a shoot call.  A CTA of WARPS warps covers WARPS consecutive grid rows by 32 * RPT
+// consecutive columns, laid out over its warps and threads as RayTile says: lane l of a warp holds
+// columns c0 + l + 32 k, k < 2 CP, of the warp's R rows.
 // ----------------------------------------------------------------------------------------------
 template <int WARPS, int RPT>
 __host__ __device__ __forceinline__ int64_t shoot_tiles(int64_t n_rows, int64_t n0) {
@@ -955,9 +1011,12 @@ __device__ __forceinline__ bool shoot_tile(const ShootDesc& d, int64_t tile, Sho
   const int64_t ncol = (d.n0 + SEG - 1) / SEG;
   const int64_t trow = tile / ncol;
   const int64_t tcol = tile - trow * ncol;
+  using RT = RayTile<RPT>;
+  static_assert(WARPS % RT::WC == 0, "whole rows of warps");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t jrel = trow * WARPS + warp;
-  const bool row_ok = jrel < d.n_rows;
+  const int row0 = warp / RT::WC * RT::R;                       // the warp's first row of the tile
+  const int col0 = warp % RT::WC * (64 * RT::CP);               // and first column
+  const int64_t jrel = trow * WARPS + row0;
   // Ray coordinates (float64 fma rounded to float, as the header defines them) of the tile's SEG
   // columns and WARPS rows, each formed once per CTA rather than once per warp: the float64 pipe is
   // narrow, and on small fields these conversions would otherwise delay every tile's start.
@@ -980,20 +1039,22 @@ __device__ __forceinline__ bool shoot_tile(const ShootDesc& d, int64_t tile, Sho
                  ray_coord(d.j_begin + ja, d.sp1, d.or1), ray_coord(d.j_begin + jb, d.sp1, d.or1));
   }
   __syncthreads();
-  const float x2r = sm.x2row[warp];
   float x1[RPT], x2[RPT];
   bool valid[RPT];
 #pragma unroll
   for (int k = 0; k < RPT; ++k) {
-    const int64_t i = tcol * SEG + lane + 32 * k;
-    valid[k] = row_ok && i < d.n0;
-    x1[k] = sm.x1col[lane + 32 * k];
-    x2[k] = x2r;
+    const int r = k / (2 * RT::CP), c = col0 + lane + 32 * (k % (2 * RT::CP));
+    valid[k] = jrel + r < d.n_rows && tcol * SEG + c < d.n0;
+    x1[k] = sm.x1col[c];
+    x2[k] = sm.x2row[row0 + r];
   }
+  // a warp past the last row or column of the call has no ray to sum (ragged grids)
+  const bool active = jrel < d.n_rows && tcol * SEG + col0 < d.n0;
   float a1h[RPT], a1l[RPT], a2h[RPT], a2l[RPT], sig[RPT], tn[RPT];
-  if (!deflect_pairs<RPT, TILE, MASS, true, WARPS>(d.f, x1, x2, a1h, a1l, a2h, a2l, sig, tn, sm, ps, &ss.near))
+  if (!deflect_pairs<RPT, TILE, MASS, true, WARPS>(d.f, x1, x2, a1h, a1l, a2h, a2l, sig, tn, sm, ps, &ss.near, active))
     return false;
-  bin_rays<RPT, 32>(d, x1, x2, a1h, a1l, a2h, a2l, sig, tn, valid, jrel, tcol * SEG + lane, lane);
+  if (active)
+    bin_rays<RPT, 2 * RT::CP, 32>(d, x1, x2, a1h, a1l, a2h, a2l, sig, tn, valid, jrel, tcol * SEG + col0 + lane, lane);
   return true;
 }
 

@@ -49,22 +49,25 @@ __global__ void __launch_bounds__(kBlock, 2) staged_kernel(const ShootDesc d, ui
   const int64_t ncol = (d.n0 + SEG - 1) / SEG;
   const int64_t trow = tile / ncol;
   const int64_t tcol = tile - trow * ncol;
+  using RT = RayTile<kRpt>;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t jrel = trow * kWarps + warp;
-  const bool row_ok = jrel < d.n_rows;
-  const int64_t j = d.j_begin + (row_ok ? jrel : d.n_rows - 1);
-  const float x2r = ray_coord(j, d.sp1, d.or1);
+  const int row0 = warp / RT::WC * RT::R, col0 = warp % RT::WC * (64 * RT::CP);
+  const int64_t jrel = trow * kWarps + row0;
   float x1[kRpt], x2[kRpt];
   bool valid[kRpt];
 #pragma unroll
   for (int k = 0; k < kRpt; ++k) {
-    int64_t i = tcol * SEG + lane + 32 * k;
-    valid[k] = row_ok && i < d.n0;
+    const int r = k / (2 * RT::CP);
+    int64_t i = tcol * SEG + col0 + lane + 32 * (k % (2 * RT::CP)), j = jrel + r;
+    valid[k] = j < d.n_rows && i < d.n0;
     if (i >= d.n0) i = d.n0 - 1;
+    if (j >= d.n_rows) j = d.n_rows - 1;
     x1[k] = ray_coord(i, d.sp0, d.or0);
-    x2[k] = x2r;
+    x2[k] = ray_coord(d.j_begin + j, d.sp1, d.or1);
+    if (lane == 0 && col0 == 0 && k % (2 * RT::CP) == 0) sm.x2row[row0 + r] = x2[k];
   }
-  if (lane == 0) sm.x2row[warp] = x2r;
+  // a warp past the last row or column of the call has no ray to sum
+  const bool active = jrel < d.n_rows && tcol * SEG + col0 < d.n0;
   if (threadIdx.x == 0) {
     const int64_t ia = tcol * SEG, ib = min(ia + SEG, d.n0) - 1;
     const int64_t ja = trow * kWarps, jb = min(ja + kWarps, d.n_rows) - 1;
@@ -85,7 +88,7 @@ __global__ void __launch_bounds__(kBlock, 2) staged_kernel(const ShootDesc d, ui
 #pragma unroll
   for (int k = 0; k < kRpt; ++k) ss.near.t[k * kBlock + threadIdx.x] = 0.f;
   __syncthreads();  // the box and the row coordinates are set
-  if (!deflect_accumulate<kRpt, rsint::kTile, MASS, true, kWarps>(d.f, X1, X2, acc, sm, ps, &ss.near)) return;
+  if (!deflect_accumulate<kRpt, rsint::kTile, MASS, true, kWarps>(d.f, X1, X2, acc, sm, ps, &ss.near, active)) return;
   float tn[kRpt];
 #pragma unroll
   for (int q = 0; q < kNp; ++q) {
@@ -100,7 +103,8 @@ __global__ void __launch_bounds__(kBlock, 2) staged_kernel(const ShootDesc d, ui
   }
   float a1h[kRpt], a1l[kRpt], a2h[kRpt], a2l[kRpt], sig[kRpt];
   deflect_finish<kRpt>(acc, a1h, a1l, a2h, a2l, sig);
-  bin_rays<kRpt, 32>(d, x1, x2, a1h, a1l, a2h, a2l, sig, tn, valid, jrel, tcol * SEG + lane, lane);
+  if (active)
+    bin_rays<kRpt, 2 * RT::CP, 32>(d, x1, x2, a1h, a1l, a2h, a2l, sig, tn, valid, jrel, tcol * SEG + col0 + lane, lane);
 }
 
 // ---- float-float re-evaluation of the listed rays, partition by partition ----------------------
