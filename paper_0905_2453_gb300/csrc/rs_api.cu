@@ -247,6 +247,11 @@ float near_cap(int64_t n_lens, float m_max) {
   return n_lens > 0 ? m_max : 0.f;
 }
 
+int mass_mode(bool weighted, float m_max) {
+  if (!weighted) return rsdev::kUnitMass;
+  return m_max <= rsdev::kMassMax ? rsdev::kMass : rsdev::kWideMass;  // NaN (device inputs): the wide kernels
+}
+
 cudaError_t launch_pack_lenses(const float* xy, const float* m, int64_t n, int64_t n_pad, float4* lens4,
                                float2* mass2, int blocks, cudaStream_t s) {
   pack_lenses_kernel<<<blocks, 256, 0, s>>>(xy, m, n, n_pad, lens4, mass2);
@@ -439,7 +444,7 @@ int rs_create_field(const float* lens_xy, const float* masses, int64_t n_lens, d
   f->dev.lens4 = f->lens4;
   f->dev.mass2 = has_mass ? f->mass2 : nullptr;
   f->dev.n_lens = (int32_t)n_lens;
-  f->dev.has_mass = (has_mass && !unit_masses) ? 1 : 0;
+  f->dev.has_mass = mass_mode(has_mass && !unit_masses, m_max);
   f->dev.lam1 = (1.0 - kappa_c) - gamma;
   f->dev.lam2 = (1.0 - kappa_c) + gamma;
   f->dev.lamabs = std::nextafter((float)std::max(std::fabs(f->dev.lam1), std::fabs(f->dev.lam2)), INFINITY);
@@ -596,7 +601,7 @@ int rs_field_time(rs_field_t f, double* t) {
 int rs_field_info(rs_field_t f, int64_t* n_lens, int* has_masses) {
   if (!f) return fail(RS_EINVAL, "field is NULL");
   if (n_lens) *n_lens = f->n_lens;
-  if (has_masses) *has_masses = f->dev.has_mass;
+  if (has_masses) *has_masses = f->dev.has_mass != rsdev::kUnitMass ? 1 : 0;
   return RS_OK;
 }
 

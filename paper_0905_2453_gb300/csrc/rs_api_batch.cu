@@ -15,8 +15,9 @@ struct rs_batch {
   int device;
   int n_fields;
   // work items grouped by (launch shape, mass mode): one persistent kernel per group; group
-  // g = 2 * cfg + mass (mass 0: unit masses, 1: per-lens masses)
-  static constexpr int kGroups = 2 * rsint::kNumCfg;
+  // g = kMassModes * cfg + mass (rsdev::MassMode)
+  static constexpr int kMassModes = 3;
+  static constexpr int kGroups = kMassModes * rsint::kNumCfg;
   int n_items[kGroups];
   int item_offset[kGroups];
   int grid[kGroups];
@@ -62,8 +63,8 @@ int rs_batch_create_shaped(int n_fields, const rs_field_t* fields, const rs_ray_
     if ((rc = fill_desc(fields[k], &grids[k], 0, grids[k].n[1], &windows[k], d_counts[k],
                         d_out_of_window ? d_out_of_window + k : nullptr, &descs[k])) != RS_OK)
       return rc;
-    const int mass = fields[k]->dev.has_mass ? 1 : 0;
-    int cfg = g_cfg[mass];
+    const int mass = fields[k]->dev.has_mass;
+    int cfg = g_cfg[mass ? 1 : 0];
     if (shapes) {
       const int* sh = shapes + 4 * k;
       cfg = rsint::find_cfg(sh[0], sh[1], sh[2], sh[3]);
@@ -71,8 +72,8 @@ int rs_batch_create_shaped(int n_fields, const rs_field_t* fields, const rs_ray_
         return fail(RS_EINVAL, "shapes[%d] = (%d, %d, %d, %d) is not a compiled launch shape", k, sh[0], sh[1], sh[2],
                     sh[3]);
     }
-    cfg = rsint::batch_cfg(cfg);
-    const int grp = 2 * cfg + mass;
+    cfg = mass == rsdev::kWideMass ? rsint::kDefaultCfg : rsint::batch_cfg(cfg);
+    const int grp = rs_batch::kMassModes * cfg + mass;
     const int warps = rsint::kCfgs[cfg].block / 32;
     const int64_t seg = 32 * (int64_t)rsint::kCfgs[cfg].rpt;
     const int64_t n0 = descs[k].n0, nr = descs[k].n_rows;
@@ -104,7 +105,7 @@ int rs_batch_create_shaped(int n_fields, const rs_field_t* fields, const rs_ray_
     b->grid[grp] = 0;
     if (b->n_items[grp] == 0) continue;
     int bps = 0;
-    if (rsint::batch_blocks_per_sm(grp / 2, (grp & 1) == 1, &bps) != cudaSuccess || bps < 1) bps = 1;
+    if (rsint::batch_blocks_per_sm(grp / rs_batch::kMassModes, grp % rs_batch::kMassModes, &bps) != cudaSuccess || bps < 1) bps = 1;
     b->grid[grp] = num_sms(dev) * bps;
   }
   auto cleanup = [&]() {
@@ -165,7 +166,7 @@ int rs_batch_create_shaped(int n_fields, const rs_field_t* fields, const rs_ray_
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return items[x][0].cost > items[y][0].cost; });
     for (size_t i = 0; i < order.size() && e == cudaSuccess; ++i) {
       const int grp = order[i];
-      e = rsint::launch_batch(grp / 2, (grp & 1) == 1, b->d_descs, b->d_items + b->item_offset[grp], b->n_items[grp],
+      e = rsint::launch_batch(grp / rs_batch::kMassModes, grp % rs_batch::kMassModes, b->d_descs, b->d_items + b->item_offset[grp], b->n_items[grp],
                               b->d_counter + grp, b->grid[grp], cs);
     }
     if (e == cudaSuccess && b->rc_cap > 0)

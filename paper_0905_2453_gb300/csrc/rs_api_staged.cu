@@ -47,7 +47,7 @@ int rs_shoot_staged(int n_parts, const rs_field_t* parts, const rs_ray_grid* g, 
   // one kernel for every partition: the weighted one if any partition has masses other than 1 (all
   // partitions then store masses)
   int weighted = 0;
-  for (int p = 0; p < n_parts; ++p) weighted |= parts[p]->dev.has_mass;
+  for (int p = 0; p < n_parts; ++p) weighted = std::max(weighted, parts[p]->dev.has_mass);
   int rc;
   if ((rc = check_call(g, row_begin, row_end, w, d_counts)) != RS_OK) return rc;
   if ((rc = check_field_device(parts[0])) != RS_OK) return rc;
@@ -132,7 +132,7 @@ int rs_shoot_streamed(const float* h_lens_xy, const float* h_masses, int64_t n_l
   proto.device = dev;
   proto.kappa_c = kappa_c;
   proto.gamma = gamma;
-  proto.dev.has_mass = mass ? 1 : 0;
+  proto.dev.has_mass = mass_mode(mass, m_max);
   proto.dev.lam1 = (1.0 - kappa_c) - gamma;
   proto.dev.lam2 = (1.0 - kappa_c) + gamma;
   proto.dev.lamabs = std::nextafter((float)std::max(std::fabs(proto.dev.lam1), std::fabs(proto.dev.lam2)), INFINITY);
@@ -312,7 +312,9 @@ int partition_desc(rs_field_t part, int weighted, const rs_ray_grid* g, int64_t 
     return fail(RS_EINVAL, "the partition's masses are not all 1: every pass of the shoot must be weighted");
   if ((rc = check_field_device(part)) != RS_OK) return rc;
   if ((rc = fill_desc(part, g, row_begin, row_end, w, d_counts, d_oow, d)) != RS_OK) return rc;
-  d->f.has_mass = weighted ? 1 : 0;
+  // a partition above the kMass bound weighs its own lenses the wide way (the other partitions may be held by
+  // other processes, which do not see its masses: their kMass terms then differ from a single field's by rounding)
+  d->f.has_mass = weighted ? std::max<int>(rsdev::kMass, part->dev.has_mass) : rsdev::kUnitMass;
   return RS_OK;
 }
 

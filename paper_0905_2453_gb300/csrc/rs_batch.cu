@@ -22,7 +22,7 @@ template <int MINB>
 constexpr int batch_minb() {
   return MINB == 3 ? 2 : MINB;
 }
-template <int WARPS, int RPT, int TILE, bool MASS, int MINB>
+template <int WARPS, int RPT, int TILE, int MASS, int MINB>
 __global__ void __launch_bounds__(WARPS * 32, MINB)
     batch_kernel(const ShootDesc* __restrict__ descs, const int2* __restrict__ items, int n_items, int* counter) {
   extern __shared__ __align__(128) unsigned char rs_smem[];
@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB)
   }
 }
 
-template <int WARPS, int RPT, int TILE, bool MASS, int MINB>
+template <int WARPS, int RPT, int TILE, int MASS, int MINB>
 cudaError_t launch_batch_m(const ShootDesc* descs, const int2* items, int n_items, int* counter, int grid,
                            cudaStream_t s) {
   constexpr size_t smem = sizeof(ShootSmem<WARPS, RPT, TILE>);
@@ -64,13 +64,13 @@ cudaError_t launch_batch_m(const ShootDesc* descs, const int2* items, int n_item
 }
 
 template <int WARPS, int RPT, int TILE, int MINB>
-cudaError_t launch_batch_t(bool mass, const ShootDesc* descs, const int2* items, int n_items, int* counter, int grid,
+cudaError_t launch_batch_t(int mass, const ShootDesc* descs, const int2* items, int n_items, int* counter, int grid,
                            cudaStream_t s) {
-  return mass ? launch_batch_m<WARPS, RPT, TILE, true, MINB>(descs, items, n_items, counter, grid, s)
-              : launch_batch_m<WARPS, RPT, TILE, false, MINB>(descs, items, n_items, counter, grid, s);
+  return mass ? launch_batch_m<WARPS, RPT, TILE, kMass, MINB>(descs, items, n_items, counter, grid, s)
+              : launch_batch_m<WARPS, RPT, TILE, kUnitMass, MINB>(descs, items, n_items, counter, grid, s);
 }
 
-template <int WARPS, int RPT, int TILE, bool MASS, int MINB>
+template <int WARPS, int RPT, int TILE, int MASS, int MINB>
 cudaError_t occ_m(int* blocks) {
   constexpr size_t smem = sizeof(ShootSmem<WARPS, RPT, TILE>);
   cudaError_t e = rsint::smem_opt_in<batch_kernel<WARPS, RPT, TILE, MASS, MINB>>(smem);
@@ -80,16 +80,19 @@ cudaError_t occ_m(int* blocks) {
 }
 
 template <int WARPS, int RPT, int TILE, int MINB>
-cudaError_t occ_t(bool mass, int* blocks) {
-  return mass ? occ_m<WARPS, RPT, TILE, true, MINB>(blocks) : occ_m<WARPS, RPT, TILE, false, MINB>(blocks);
+cudaError_t occ_t(int mass, int* blocks) {
+  return mass ? occ_m<WARPS, RPT, TILE, kMass, MINB>(blocks) : occ_m<WARPS, RPT, TILE, kUnitMass, MINB>(blocks);
 }
 
 }  // namespace
 
 namespace rsint {
 
-cudaError_t launch_batch(int cfg, bool mass, const rsdev::ShootDesc* descs, const int2* items, int n_items,
+cudaError_t launch_batch(int cfg, int mass, const rsdev::ShootDesc* descs, const int2* items, int n_items,
                          int* counter, int grid, cudaStream_t s) {
+  if (mass == rsdev::kWideMass)
+    return launch_batch_m<kWideWarps, kWideRpt, kWideTile, rsdev::kWideMass, 2>(descs, items, n_items, counter, grid,
+                                                                                s);
   switch (cfg) {
 #define RS_CASE(i, w, r, t, m) \
   case i:                       \
@@ -100,7 +103,8 @@ cudaError_t launch_batch(int cfg, bool mass, const rsdev::ShootDesc* descs, cons
   }
 }
 
-cudaError_t batch_blocks_per_sm(int cfg, bool mass, int* blocks) {
+cudaError_t batch_blocks_per_sm(int cfg, int mass, int* blocks) {
+  if (mass == rsdev::kWideMass) return occ_m<kWideWarps, kWideRpt, kWideTile, rsdev::kWideMass, 2>(blocks);
   switch (cfg) {
 #define RS_CASE(i, w, r, t, m) \
   case i:                       \

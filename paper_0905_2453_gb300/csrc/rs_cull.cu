@@ -44,7 +44,7 @@ __device__ __forceinline__ void fold(float& hi, float& lo, float p) {
 // cell's source-plane box against the window.  Kept cells are appended to `out`; skipped cells add
 // their rays to the out-of-window count.  Two levels: cells of 64 x 64 rays over the whole call
 // (parent == nullptr), then the 16 cells of 16 x 16 rays of every kept 64 x 64 cell.
-template <bool MASS>
+template <int MASS>
 __global__ void __launch_bounds__(kCullBlock)
     cull_kernel(const ShootDesc d, int cell_rays, int64_t n_cx, int64_t n_cells, const unsigned* __restrict__ parent,
                 const unsigned* __restrict__ parent_count, int64_t n_px, double hi0, double hi1,
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kCullBlock)
 // Kept cells: a CTA of four warps shoots four cells per pass (one per warp); lane l holds row l / 2
 // of its cell and columns 8 (l % 2) .. 8 (l % 2) + 7.  The per-ray arithmetic is rs_shoot's (per-ray
 // squared distances instead of the shared row table give bitwise the same values).
-template <bool MASS>
+template <int MASS>
 __global__ void __launch_bounds__(128, 2) shoot_cells_kernel(const ShootDesc d, int64_t n_cx,
                                                              const unsigned* __restrict__ list,
                                                              const unsigned* __restrict__ n_kept) {
@@ -237,10 +237,12 @@ cudaError_t launch_cull(const rsdev::ShootDesc& d, double hi0, double hi1, unsig
 
 cudaError_t launch_shoot_cells(const rsdev::ShootDesc& d, int64_t n_cx, const unsigned* list, const unsigned* n_kept,
                                int grid, cudaStream_t s) {
-  if (d.f.has_mass)
-    shoot_cells_kernel<true><<<grid, 128, 0, s>>>(d, n_cx, list, n_kept);
+  if (d.f.has_mass == rsdev::kWideMass)
+    shoot_cells_kernel<rsdev::kWideMass><<<grid, 128, 0, s>>>(d, n_cx, list, n_kept);
+  else if (d.f.has_mass)
+    shoot_cells_kernel<rsdev::kMass><<<grid, 128, 0, s>>>(d, n_cx, list, n_kept);
   else
-    shoot_cells_kernel<false><<<grid, 128, 0, s>>>(d, n_cx, list, n_kept);
+    shoot_cells_kernel<rsdev::kUnitMass><<<grid, 128, 0, s>>>(d, n_cx, list, n_kept);
   return cudaGetLastError();
 }
 

@@ -17,7 +17,7 @@
 //     and its square come from a per-row table built in shared memory once per
 //     lens tile, and (x1 - x1_lens) of a column pair serves both its rows.
 //   * Per lens and ray pair: half a sub.f32x2, fma.f32x2 (|d|^2), the reciprocal,
-//     [mul.f32x2 by the mass], fma.f32x2 x2 -- the ten flops per interaction of
+//     fma.f32x2 x2 (masses: half a mul.f32x2 more, they multiply the distances) -- the ten flops per interaction of
 //     the paper's Appendix A.  For three of every four lens pairs (unit masses;
 //     one of two with masses) one rcp.approx of the product of the two squared
 //     distances serves both lenses (Montgomery's simultaneous inversion), which
@@ -180,11 +180,23 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 // ----------------------------------------------------------------------------------------------
 // Descriptors.
 // ----------------------------------------------------------------------------------------------
+// How a field's kernels weigh the lenses (template parameter MASS).
+//   kUnitMass  every m = 1: no mass is read.
+//   kMass      the mass multiplies the distances, P += w (m d) with w = 1 / r^2: m d2 sits in the row
+//              table and m d1 serves all rows of a thread, so a lens costs half a packed multiply per ray
+//              pair instead of one.
+//   kWideMass  the mass multiplies w, P += (m w) d: fields with a mass above 2^64, whose m d could
+//              overflow where m w d does not (|d| < 2^32: below 2^64 there are 2^32 to spare).  Downwards
+//              m d is flushed only below 1.2e-38, a term m / d that is seen next to a coordinate of order 1
+//              only at d < 1e-19, where r^2 itself is flushed.
+enum MassMode : int { kUnitMass = 0, kMass = 1, kWideMass = 2 };
+constexpr float kMassMax = 0x1p64f;  // the largest mass of kMass
+
 struct FieldDev {
   const float4* lens4;  // {x1, x1, x2, x2} per lens, padded to a multiple of kLensPad lenses
   const float2* mass2;  // {m, m} per lens (same padding), or nullptr for unit masses
   int32_t n_lens;
-  int32_t has_mass;
+  int32_t has_mass;     // MassMode
   double lam1, lam2;    // (1 - kappa_c) - gamma, (1 - kappa_c) + gamma
   float lamabs;         // max(|lam1|, |lam2|), for the Eq. 6 rounding term of the error band
   float mcap;           // the largest mass / h: bounds every term of a lens farther than h from a ray (0: no lenses)
@@ -319,7 +331,7 @@ __device__ __forceinline__ void near_gather(NS& ns, int par, const float4* l4, i
 
 // Near terms of group g's lenses listed with parity par for the thread's rays (packed pairs X1, X2),
 // folded into the thread's entries of ns.t; lens coordinates from the field's arrays.
-template <int NP, bool MASS, class NS>
+template <int NP, int MASS, class NS>
 __device__ __forceinline__ void near_eval(NS& ns, int par, int g, const FieldDev& f, const uint64_t (&X1)[NP],
                                           const uint64_t (&X2)[NP], int nthreads) {
   const int n = ns.n[par][g];
@@ -344,7 +356,7 @@ __device__ __forceinline__ void near_eval(NS& ns, int par, int g, const FieldDev
 }
 
 // T of one ray over every lens of a field (listed-ray kernels): the same value as the shoot's.
-template <bool MASS>
+template <int MASS>
 __device__ __forceinline__ float near_term_all(const FieldDev& f, float x1, float x2) {
   float t = f.mcap;
   for (int l = 0; l < f.n_lens; ++l) {
@@ -359,7 +371,7 @@ template <int TILE, int ROWS = 1>
 struct __align__(16) LensSmem {
   float4 lens4[2][TILE];     // double-buffered lens tiles {x1, x1, x2, x2}
   float2 mass2[2][TILE];     // {m, m}
-  float4 rowtab[ROWS][TILE]; // per CTA row r and lens l of the current tile: {d2, d2, d2^2, d2^2}
+  float4 rowtab[ROWS][TILE]; // per CTA row r and lens l of the current tile: {E2, E2, d2^2, d2^2}
   float2 x1tab[ROWS > 1 ? TILE : 2];  // {x1, x1} of the current tile's lenses: a lens pair in one 16-byte load
   float x2row[ROWS];         // x2 of the CTA's rows
   float x1col[kMaxSeg];      // x1 of the CTA's columns (shoot_tile)
@@ -382,7 +394,7 @@ __device__ __forceinline__ void pipe_init(uint64_t* bar, PipeState& ps) {
   __syncthreads();
 }
 
-template <int TILE, bool MASS, int ROWS>
+template <int TILE, int MASS, int ROWS>
 __device__ __forceinline__ void issue_lens_tile(const FieldDev& f, LensSmem<TILE, ROWS>& sm, int tile, int buf) {
   // called by one thread.  The tile's lenses rounded up to an even count (16-byte multiples for both
   // arrays): at most one lens past the field's last, which the padding of the device arrays (and of a
@@ -406,7 +418,8 @@ __device__ __forceinline__ float ray_coord(int64_t idx, double spacing, double o
 
 // ----------------------------------------------------------------------------------------------
 // Lens-pair step.  Two consecutive lenses a, b against one ray pair (lanes A, B of each operand).
-// With d1 = x1 - x1_lens, d2 and d2^2 (S2) supplied: r2 = d1^2 + d2^2; w = m / r2; P += w * (d1, d2).
+// With d1 = x1 - x1_lens and d2^2 (S2) supplied: r2 = d1^2 + d2^2, w = 1 / r2 (kWideMass: m / r2),
+// P += w * (E1, E2) with (E1, E2) the distances as weigh leaves them.
 //
 // MONT: one reciprocal serves both lenses (Montgomery's simultaneous inversion):
 //   inv = 1 / (r2a * r2b),  1/r2a = r2b * inv,  1/r2b = r2a * inv.
@@ -415,9 +428,10 @@ __device__ __forceinline__ float ray_coord(int64_t idx, double spacing, double o
 // only underflow when the ray is within ~3e-10 of one of the two lenses, a ray whose own
 // deflection is then ~1e9 (out of any window), and only that ray is affected.
 // ----------------------------------------------------------------------------------------------
-template <bool MONT, bool MASS>
-__device__ __forceinline__ void lens_pair_step(uint64_t d1a, uint64_t d1b, uint64_t D2a, uint64_t S2a, uint64_t D2b,
-                                               uint64_t S2b, uint64_t Ma, uint64_t Mb, uint64_t& P1, uint64_t& P2) {
+template <bool MONT, int MASS>
+__device__ __forceinline__ void lens_pair_step(uint64_t d1a, uint64_t d1b, uint64_t E1a, uint64_t E1b, uint64_t E2a,
+                                               uint64_t S2a, uint64_t E2b, uint64_t S2b, uint64_t Ma, uint64_t Mb,
+                                               uint64_t& P1, uint64_t& P2) {
   const uint64_t r2a = f2_fma(d1a, d1a, S2a);
   const uint64_t r2b = f2_fma(d1b, d1b, S2b);
   uint64_t wa, wb;
@@ -435,40 +449,47 @@ __device__ __forceinline__ void lens_pair_step(uint64_t d1a, uint64_t d1b, uint6
     wa = f2_pack(rcp_approx(a0), rcp_approx(a1));
     wb = f2_pack(rcp_approx(b0), rcp_approx(b1));
   }
-  if (MASS) {
+  if (MASS == kWideMass) {
     wa = f2_mul(wa, Ma);
     wb = f2_mul(wb, Mb);
   }
-  P1 = f2_fma(wa, d1a, P1);
-  P2 = f2_fma(wa, D2a, P2);
-  P1 = f2_fma(wb, d1b, P1);
-  P2 = f2_fma(wb, D2b, P2);
+  P1 = f2_fma(wa, E1a, P1);
+  P2 = f2_fma(wa, E2a, P2);
+  P1 = f2_fma(wb, E1b, P1);
+  P2 = f2_fma(wb, E2b, P2);
+}
+
+// A distance as the accumulation takes it: weighed by the mass with kMass.
+template <int MASS>
+__device__ __forceinline__ uint64_t weigh(uint64_t d, uint64_t M) {
+  return MASS == kMass ? f2_mul(d, M) : d;
 }
 
 // A single lens (the odd last lens of a field), direct reciprocal.
-template <bool MASS>
-__device__ __forceinline__ void lens_single_step(uint64_t d1, uint64_t D2, uint64_t S2, uint64_t M, uint64_t& P1,
-                                                 uint64_t& P2) {
+template <int MASS>
+__device__ __forceinline__ void lens_single_step(uint64_t d1, uint64_t E1, uint64_t E2, uint64_t S2, uint64_t M,
+                                                 uint64_t& P1, uint64_t& P2) {
   const uint64_t r2 = f2_fma(d1, d1, S2);
   float a0, a1;
   f2_unpack(r2, a0, a1);
   uint64_t w = f2_pack(rcp_approx(a0), rcp_approx(a1));
-  if (MASS) w = f2_mul(w, M);
-  P1 = f2_fma(w, d1, P1);
-  P2 = f2_fma(w, D2, P2);
+  if (MASS == kWideMass) w = f2_mul(w, M);
+  P1 = f2_fma(w, E1, P1);
+  P2 = f2_fma(w, E2, P2);
 }
 
 // Which lens pairs of a group use the shared reciprocal: pair index p within its group.
-// Unit masses: three of every four pairs; per-lens masses (one more multiply per lens): every
-// other pair.  These ratios balance the FMA and MUFU pipes; they are fixed, so every ray of a
-// field always gets the same arithmetic.
-template <bool MASS>
+// Unit masses: three of every four pairs; per-lens masses (more multiplies per lens): every other
+// pair.  These ratios balance the FMA and MUFU pipes (body alone on 1e4 lenses, 4096^2 rays: unit
+// masses 3/4 27.7 ms, 5/8 27.8, 1/2 28.1, 7/8 28.3; masses 1/2 29.7 ms, 5/8 29.9, 3/4 30.3, 3/8 30.7);
+// they are fixed, so every ray of a field always gets the same arithmetic.
+template <int MASS>
 __device__ __forceinline__ constexpr bool mont_pair(int p) {
   return MASS ? ((p & 1) == 0) : ((p & 3) != 3);
 }
 
 // Loads lens l of the current shared-memory buffer: Lx = {x1, x1}, Ly = {x2, x2}, M = {m, m}.
-template <bool MASS>
+template <int MASS>
 __device__ __forceinline__ void load_lens(uint32_t lbase, uint32_t mbase, int l, uint64_t& Lx, uint64_t& Ly,
                                           uint64_t& M) {
   lds_pair2(lbase + (uint32_t)l * 16u, Lx, Ly);
@@ -477,7 +498,7 @@ __device__ __forceinline__ void load_lens(uint32_t lbase, uint32_t mbase, int l,
 
 // One lens pair (lenses l, l + 1) against all ray pairs of the thread, every ray pair with its own
 // x2 (listed rays, cells): d2 and d2^2 are formed per ray pair.
-template <int NP, bool MONT, bool MASS>
+template <int NP, bool MONT, int MASS>
 __device__ __forceinline__ void lens_pair_all(uint32_t lbase, uint32_t mbase, int l, const uint64_t (&X1)[NP],
                                               const uint64_t (&X2)[NP], uint64_t (&P1)[NP], uint64_t (&P2)[NP]) {
   uint64_t Lxa, Lya, Ma, Lxb, Lyb, Mb;
@@ -487,7 +508,9 @@ __device__ __forceinline__ void lens_pair_all(uint32_t lbase, uint32_t mbase, in
   for (int q = 0; q < NP; ++q) {
     const uint64_t D2a = f2_sub(X2[q], Lya), D2b = f2_sub(X2[q], Lyb);
     const uint64_t S2a = f2_mul(D2a, D2a), S2b = f2_mul(D2b, D2b);
-    lens_pair_step<MONT, MASS>(f2_sub(X1[q], Lxa), f2_sub(X1[q], Lxb), D2a, S2a, D2b, S2b, Ma, Mb, P1[q], P2[q]);
+    const uint64_t d1a = f2_sub(X1[q], Lxa), d1b = f2_sub(X1[q], Lxb);
+    lens_pair_step<MONT, MASS>(d1a, d1b, weigh<MASS>(d1a, Ma), weigh<MASS>(d1b, Mb), weigh<MASS>(D2a, Ma), S2a,
+                               weigh<MASS>(D2b, Mb), S2b, Ma, Mb, P1[q], P2[q]);
   }
 }
 
@@ -502,24 +525,26 @@ __device__ __forceinline__ void lens_pair_all(uint32_t lbase, uint32_t mbase, in
 // 5.125.  Body alone, 1e4 unit-mass lenses, 4096^2 rays: one row of eight columns 29.6 ms, two rows of
 // four 27.7 ms; four rows of four (16 rays per thread) 27.4 ms but with half the warps to cover a CTA's
 // start and end, so two rows are kept.
-template <int R, int CP, int TILE, bool MONT, bool MASS>
+template <int R, int CP, int TILE, bool MONT, int MASS>
 __device__ __forceinline__ void lens_pair_rows(uint32_t xbase, uint32_t mbase, uint32_t rt, int l,
                                                const uint64_t (&X1)[R * CP], uint64_t (&P1)[R * CP],
                                                uint64_t (&P2)[R * CP]) {
-  uint64_t Lxa, Lxb, Ma = 0ull, Mb = 0ull, D2a[R], S2a[R], D2b[R], S2b[R];
+  uint64_t Lxa, Lxb, Ma = 0ull, Mb = 0ull, E2a[R], S2a[R], E2b[R], S2b[R];
   lds_pair2(xbase + (uint32_t)l * 8u, Lxa, Lxb);  // l is even: 16-byte aligned
   if (MASS) lds_pair2(mbase + (uint32_t)l * 8u, Ma, Mb);
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    lds_pair2(rt + (uint32_t)(r * TILE + l) * 16u, D2a[r], S2a[r]);
-    lds_pair2(rt + (uint32_t)(r * TILE + l + 1) * 16u, D2b[r], S2b[r]);
+    lds_pair2(rt + (uint32_t)(r * TILE + l) * 16u, E2a[r], S2a[r]);
+    lds_pair2(rt + (uint32_t)(r * TILE + l + 1) * 16u, E2b[r], S2b[r]);
   }
 #pragma unroll
   for (int c = 0; c < CP; ++c) {
     const uint64_t d1a = f2_sub(X1[c], Lxa), d1b = f2_sub(X1[c], Lxb);
+    const uint64_t E1a = weigh<MASS>(d1a, Ma), E1b = weigh<MASS>(d1b, Mb);
 #pragma unroll
     for (int r = 0; r < R; ++r)
-      lens_pair_step<MONT, MASS>(d1a, d1b, D2a[r], S2a[r], D2b[r], S2b[r], Ma, Mb, P1[r * CP + c], P2[r * CP + c]);
+      lens_pair_step<MONT, MASS>(d1a, d1b, E1a, E1b, E2a[r], S2a[r], E2b[r], S2b[r], Ma, Mb, P1[r * CP + c],
+                                 P2[r * CP + c]);
   }
 }
 
@@ -533,7 +558,7 @@ struct RayTile {
   static constexpr int WC = R;
 };
 
-template <int RPT, int TILE, bool MONT, bool MASS, bool ROW>
+template <int RPT, int TILE, bool MONT, int MASS, bool ROW>
 __device__ __forceinline__ void lens_pair_any(uint32_t lbase, uint32_t xbase, uint32_t mbase, uint32_t rt, int l,
                                               const uint64_t (&X1)[RPT / 2], const uint64_t (&X2)[RPT / 2],
                                               uint64_t (&P1)[RPT / 2], uint64_t (&P2)[RPT / 2]) {
@@ -544,7 +569,7 @@ __device__ __forceinline__ void lens_pair_any(uint32_t lbase, uint32_t xbase, ui
 }
 
 // Four lens pairs of a group (lenses l .. l + 7, l a multiple of 8 within the group): the fixed reciprocal pattern.
-template <int RPT, int TILE, bool MASS, bool ROW>
+template <int RPT, int TILE, int MASS, bool ROW>
 __device__ __forceinline__ void lens_block(uint32_t lbase, uint32_t xbase, uint32_t mbase, uint32_t rt, int l,
                                            const uint64_t (&X1)[RPT / 2], const uint64_t (&X2)[RPT / 2],
                                            uint64_t (&P1)[RPT / 2], uint64_t (&P2)[RPT / 2]) {
@@ -556,7 +581,7 @@ __device__ __forceinline__ void lens_block(uint32_t lbase, uint32_t xbase, uint3
 
 // The last, partial group of a field (cnt < 64 lenses from l0): the same pattern by pair index, an odd last
 // lens directly.
-template <int RPT, int TILE, bool MASS, bool ROW>
+template <int RPT, int TILE, int MASS, bool ROW>
 __device__ __forceinline__ void lens_group_partial(uint32_t lbase, uint32_t xbase, uint32_t mbase, uint32_t rt, int l0,
                                                    int cnt, const uint64_t (&X1)[RPT / 2],
                                                    const uint64_t (&X2)[RPT / 2], uint64_t (&P1)[RPT / 2],
@@ -578,38 +603,41 @@ __device__ __forceinline__ void lens_group_partial(uint32_t lbase, uint32_t xbas
       constexpr int R = RayTile<RPT>::R, CP = RayTile<RPT>::CP;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        uint64_t D2, S2;
-        lds_pair2(rt + (uint32_t)(r * TILE + l) * 16u, D2, S2);
+        uint64_t E2, S2;
+        lds_pair2(rt + (uint32_t)(r * TILE + l) * 16u, E2, S2);
 #pragma unroll
-        for (int c = 0; c < CP; ++c)
-          lens_single_step<MASS>(f2_sub(X1[c], Lx), D2, S2, M, P1[r * CP + c], P2[r * CP + c]);
+        for (int c = 0; c < CP; ++c) {
+          const uint64_t d1 = f2_sub(X1[c], Lx);
+          lens_single_step<MASS>(d1, weigh<MASS>(d1, M), E2, S2, M, P1[r * CP + c], P2[r * CP + c]);
+        }
       }
     } else {
 #pragma unroll
       for (int q = 0; q < RPT / 2; ++q) {
-        const uint64_t D2 = f2_sub(X2[q], Ly);
-        lens_single_step<MASS>(f2_sub(X1[q], Lx), D2, f2_mul(D2, D2), M, P1[q], P2[q]);
+        const uint64_t D2 = f2_sub(X2[q], Ly), d1 = f2_sub(X1[q], Lx);
+        lens_single_step<MASS>(d1, weigh<MASS>(d1, M), weigh<MASS>(D2, M), f2_mul(D2, D2), M, P1[q], P2[q]);
       }
     }
   }
 }
 
-// Row table for the current lens tile: entry (r, l) = {d2, d2, d2^2, d2^2} with d2 = x2(row r) - x2(lens l),
-// the same float32 operations a thread would otherwise repeat for every lens.
+// Row table for the current lens tile: entry (r, l) = {E2, E2, d2^2, d2^2} with d2 = x2(row r) - x2(lens l) and
+// E2 = d2 as weigh leaves it, the same float32 operations a thread would otherwise repeat for every lens.
 // (Only the tile's cnt lenses: the last tile of a small field may hold far fewer than TILE.)
-template <int TILE, int ROWS>
+template <int MASS, int TILE, int ROWS>
 __device__ __forceinline__ void build_row_table(LensSmem<TILE, ROWS>& sm, int b, int cnt) {
   constexpr int BLOCK = ROWS * 32;
   for (int l = threadIdx.x; l < cnt; l += BLOCK) {
     const float4 L = sm.lens4[b][l];
     const float y = L.z;
     sm.x1tab[l] = make_float2(L.x, L.x);
+    const float m = MASS == kMass ? sm.mass2[b][l].x : 1.f;
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
       const uint64_t D2 = f2_sub(f2_pack(sm.x2row[r], sm.x2row[r]), f2_pack(y, y));
       const uint64_t S2 = f2_mul(D2, D2);
       float d0, d1, s0, s1;
-      f2_unpack(D2, d0, d1);
+      f2_unpack(weigh<MASS>(D2, f2_pack(m, m)), d0, d1);
       f2_unpack(S2, s0, s1);
       sm.rowtab[r][l] = make_float4(d0, d1, s0, s1);
     }
@@ -651,7 +679,7 @@ __device__ __forceinline__ void fold_group(DeflectAcc<NP>& a, const uint64_t (&P
 // With a near-lens search (NS::kOn), every tile's lenses inside the group boxes of ns are listed and
 // their near terms folded into ns.t (the caller sets the boxes and the thread's ns.t entries).  A warp
 // without a ray of the call (active false, warp-uniform) takes part in the copies, tables and barriers only.
-template <int RPT, int TILE, bool MASS, bool ROW, int ROWS, class NS = NoNear>
+template <int RPT, int TILE, int MASS, bool ROW, int ROWS, class NS = NoNear>
 __device__ __forceinline__ bool deflect_accumulate(const FieldDev& f, const uint64_t (&X1)[RPT / 2],
                                                    const uint64_t (&X2)[RPT / 2], DeflectAcc<RPT / 2>& acc,
                                                    LensSmem<TILE, ROWS>& sm, PipeState& ps, NS* ns = nullptr,
@@ -680,7 +708,7 @@ __device__ __forceinline__ bool deflect_accumulate(const FieldDev& f, const uint
     }
     const int cnt = min(TILE, n - t * TILE);
     if (ROW) {
-      build_row_table<TILE, ROWS>(sm, b, cnt);
+      build_row_table<MASS, TILE, ROWS>(sm, b, cnt);
       __syncthreads();
     }
     if constexpr (NS::kOn) {
@@ -775,7 +803,7 @@ __device__ __forceinline__ void pack_rays(const float (&x1)[RPT], const float (&
 
 // Deflection of the thread's rays and, with a near-lens search (the caller set the boxes), the
 // largest-term bound T of every ray (tn); without one, tn = mcap (the caller adds the near terms).
-template <int RPT, int TILE, bool MASS, bool ROW, int ROWS, class NS = NoNear>
+template <int RPT, int TILE, int MASS, bool ROW, int ROWS, class NS = NoNear>
 __device__ __forceinline__ bool deflect_pairs(const FieldDev& f, const float (&x1)[RPT], const float (&x2)[RPT],
                                               float (&a1h)[RPT], float (&a1l)[RPT], float (&a2h)[RPT],
                                               float (&a2l)[RPT], float (&sig)[RPT], float (&tn)[RPT],
@@ -805,7 +833,7 @@ __device__ __forceinline__ bool deflect_pairs(const FieldDev& f, const float (&x
 }
 
 // As deflect_pairs without a near-lens search, with alpha in float64 (hi + lo, exact).
-template <int RPT, int TILE, bool MASS, bool ROW, int ROWS>
+template <int RPT, int TILE, int MASS, bool ROW, int ROWS>
 __device__ __forceinline__ bool deflect(const FieldDev& f, const float (&x1)[RPT], const float (&x2)[RPT],
                                         double (&a1)[RPT], double (&a2)[RPT], float (&sig)[RPT],
                                         LensSmem<TILE, ROWS>& sm, PipeState& ps) {
@@ -1002,7 +1030,7 @@ struct ShootSmem {
   NearSmem<TILE, 1, WARPS * 32, RPT> near;
 };
 
-template <int WARPS, int RPT, int TILE, bool MASS>
+template <int WARPS, int RPT, int TILE, int MASS>
 __device__ __forceinline__ bool shoot_tile(const ShootDesc& d, int64_t tile, ShootSmem<WARPS, RPT, TILE>& ss,
                                            PipeState& ps) {
   LensSmem<TILE, WARPS>& sm = ss.lens;

@@ -104,6 +104,8 @@ int fill_desc(const rs_field* f, const rs_ray_grid* g, int64_t row_begin, int64_
               uint32_t* d_counts, uint64_t* d_oow, rsdev::ShootDesc* d);
 // The field's cap on the term m / r of any lens farther than the near radius from a ray (0 without lenses).
 float near_cap(int64_t n_lens, float m_max);
+// rsdev::MassMode of a field whose lenses are (not) weighted by masses of at most m_max.
+int mass_mode(bool weighted, float m_max);
 // Repack n lenses (xy interleaved, m or null) into the padded layout of n_pad entries.
 cudaError_t launch_pack_lenses(const float* xy, const float* m, int64_t n, int64_t n_pad, float4* lens4,
                                float2* mass2, int blocks, cudaStream_t s);

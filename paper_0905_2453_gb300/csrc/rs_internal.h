@@ -36,6 +36,11 @@ constexpr KernelCfg kCfgs[] = {RS_LAUNCH_SHAPES(RS_CFG_ENTRY)};
 #undef RS_CFG_ENTRY
 constexpr int kNumCfg = (int)(sizeof(kCfgs) / sizeof(kCfgs[0]));
 constexpr int kDefaultCfg = 8;  // 128 threads x 8 rays x 512-lens tiles, two CTAs per SM
+// Fields of kWideMass run one shape whatever is set: the default one.
+constexpr int kWideWarps = 4, kWideRpt = 8, kWideTile = 512;
+static_assert(kCfgs[kDefaultCfg].block == 32 * kWideWarps && kCfgs[kDefaultCfg].rpt == kWideRpt &&
+                  kCfgs[kDefaultCfg].tile == kWideTile && kCfgs[kDefaultCfg].min_ctas == 2,
+              "the wide-mass kernels are the default shape's");
 
 // Dynamic shared memory beyond 48 KiB per CTA needs a one-time opt-in per kernel and device.
 template <auto Kernel>
@@ -93,10 +98,10 @@ inline unsigned int recheck_capacity(int64_t n_rays) {
 }
 
 // Persistent batched launch over LPT-ordered (field, ray tile) items.
-// mass: the items all belong to fields with (true) or without (false) per-lens masses.
-cudaError_t launch_batch(int cfg, bool mass, const rsdev::ShootDesc* descs, const int2* items, int n_items,
+// mass: the rsdev::MassMode of the items' fields (kWideMass with kDefaultCfg only).
+cudaError_t launch_batch(int cfg, int mass, const rsdev::ShootDesc* descs, const int2* items, int n_items,
                          int* counter, int grid, cudaStream_t s);
-cudaError_t batch_blocks_per_sm(int cfg, bool mass, int* blocks);
+cudaError_t batch_blocks_per_sm(int cfg, int mass, int* blocks);
 
 // Culled shooting (rs_cull.cu): cells of 16 x 16 rays, bounded first in groups of 4 x 4 cells.
 // cull_cells returns the number of 16 x 16 cells of a call (and the cells per row), cull_coarse_cells

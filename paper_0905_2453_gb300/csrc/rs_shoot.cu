@@ -8,7 +8,7 @@ using namespace rsdev;
 // MINB resident CTAs per SM as the occupancy floor: two let the compiler keep a small CTA's eight rays
 // per thread, their two-float accumulators and a deep instruction window in up to 255 registers;
 // three (168 registers) hide more latency with twelve warps per SM; eight-warp CTAs take one.
-template <int WARPS, int RPT, int TILE, bool MASS, int MINB>
+template <int WARPS, int RPT, int TILE, int MASS, int MINB>
 __global__ void __launch_bounds__(WARPS * 32, MINB) shoot_kernel(const ShootDesc d) {
   extern __shared__ __align__(128) unsigned char rs_smem[];
   auto& ss = *reinterpret_cast<ShootSmem<WARPS, RPT, TILE>*>(rs_smem);
@@ -17,7 +17,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) shoot_kernel(const ShootDesc
   (void)shoot_tile<WARPS, RPT, TILE, MASS>(d, (int64_t)blockIdx.x, ss, ps);
 }
 
-template <int BLOCK, int RPT, int TILE, bool MASS>
+template <int BLOCK, int RPT, int TILE, int MASS>
 __global__ void __launch_bounds__(BLOCK)
     trace_kernel(const FieldDev f, double or0, double or1, double sp0, double sp1, const int64_t* __restrict__ ij,
                  int64_t k, double* __restrict__ y, double* __restrict__ alpha, double* __restrict__ err) {
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(BLOCK)
   }
 }
 
-template <int WARPS, int RPT, int TILE, bool MASS, int MINB>
+template <int WARPS, int RPT, int TILE, int MASS, int MINB>
 cudaError_t launch_shoot_m(const ShootDesc& d, int64_t grid, cudaStream_t s) {
   constexpr size_t smem = sizeof(ShootSmem<WARPS, RPT, TILE>);
   cudaError_t e = rsint::smem_opt_in<shoot_kernel<WARPS, RPT, TILE, MASS, MINB>>(smem);
@@ -75,11 +75,11 @@ cudaError_t launch_shoot_t(const ShootDesc& d, cudaStream_t s) {
   const int64_t grid = shoot_tiles<WARPS, RPT>(d.n_rows, d.n0);
   if (grid <= 0) return cudaSuccess;
   if (grid >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
-  return d.f.has_mass ? launch_shoot_m<WARPS, RPT, TILE, true, MINB>(d, grid, s)
-                      : launch_shoot_m<WARPS, RPT, TILE, false, MINB>(d, grid, s);
+  return d.f.has_mass ? launch_shoot_m<WARPS, RPT, TILE, kMass, MINB>(d, grid, s)
+                      : launch_shoot_m<WARPS, RPT, TILE, kUnitMass, MINB>(d, grid, s);
 }
 
-template <int WARPS, int RPT, int TILE, bool MASS, int MINB>
+template <int WARPS, int RPT, int TILE, int MASS, int MINB>
 cudaError_t occupancy_m(int* blocks) {
   constexpr size_t smem = sizeof(ShootSmem<WARPS, RPT, TILE>);
   cudaError_t e = rsint::smem_opt_in<shoot_kernel<WARPS, RPT, TILE, MASS, MINB>>(smem);
@@ -90,7 +90,8 @@ cudaError_t occupancy_m(int* blocks) {
 
 template <int WARPS, int RPT, int TILE, int MINB>
 cudaError_t occupancy_t(bool mass, int* blocks) {
-  return mass ? occupancy_m<WARPS, RPT, TILE, true, MINB>(blocks) : occupancy_m<WARPS, RPT, TILE, false, MINB>(blocks);
+  return mass ? occupancy_m<WARPS, RPT, TILE, kMass, MINB>(blocks)
+              : occupancy_m<WARPS, RPT, TILE, kUnitMass, MINB>(blocks);
 }
 
 }  // namespace
@@ -109,6 +110,12 @@ cudaError_t shoot_blocks_per_sm(int cfg, bool mass, int* blocks) {
 }
 
 cudaError_t launch_shoot(int cfg, const rsdev::ShootDesc& d, cudaStream_t s) {
+  if (d.f.has_mass == rsdev::kWideMass) {  // built for the default shape only
+    const int64_t grid = rsdev::shoot_tiles<kWideWarps, kWideRpt>(d.n_rows, d.n0);
+    if (grid <= 0) return cudaSuccess;
+    if (grid >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
+    return launch_shoot_m<kWideWarps, kWideRpt, kWideTile, rsdev::kWideMass, 2>(d, grid, s);
+  }
   switch (cfg) {
 #define RS_CASE(i, w, r, t, m) \
   case i:                       \
@@ -124,10 +131,13 @@ cudaError_t launch_trace(const rsdev::FieldDev& f, double or0, double or1, doubl
   constexpr int B = 128, R = 4;
   if (k <= 0) return cudaSuccess;
   const int64_t grid = (k + B * R - 1) / (B * R);
-  if (f.has_mass)
-    trace_kernel<B, R, kTile, true><<<(unsigned)grid, B, 0, s>>>(f, or0, or1, sp0, sp1, ij, k, y, alpha, err);
+  if (f.has_mass == rsdev::kWideMass)
+    trace_kernel<B, R, kTile, rsdev::kWideMass>
+        <<<(unsigned)grid, B, 0, s>>>(f, or0, or1, sp0, sp1, ij, k, y, alpha, err);
+  else if (f.has_mass)
+    trace_kernel<B, R, kTile, rsdev::kMass><<<(unsigned)grid, B, 0, s>>>(f, or0, or1, sp0, sp1, ij, k, y, alpha, err);
   else
-    trace_kernel<B, R, kTile, false><<<(unsigned)grid, B, 0, s>>>(f, or0, or1, sp0, sp1, ij, k, y, alpha, err);
+    trace_kernel<B, R, kTile, rsdev::kUnitMass><<<(unsigned)grid, B, 0, s>>>(f, or0, or1, sp0, sp1, ij, k, y, alpha, err);
   return cudaGetLastError();
 }
 

@@ -36,7 +36,7 @@ __device__ __forceinline__ void state_io(uint64_t* __restrict__ st, DeflectAcc<k
 
 using StagedSmem = ShootSmem<kWarps, kRpt, rsint::kTile>;
 
-template <bool MASS>
+template <int MASS>
 __global__ void __launch_bounds__(kBlock, 2) staged_kernel(const ShootDesc d, uint64_t* __restrict__ state, int first,
                                                            int last) {
   extern __shared__ __align__(128) unsigned char rs_smem[];
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kBlock, 2) staged_kernel(const ShootDesc d, ui
 // Partial float-float deflection of each listed ray by one partition, added to ff[e] = {A1h, A1l,
 // A2h, A2l} (set on the first partition).  W warps per listed ray (see ff_warps), lanes split the
 // partition's lenses, fixed reduction order.
-template <int W, bool MASS>
+template <int W, int MASS>
 __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) recheck_part_kernel(const ShootDesc d,
                                                                                const uint2* __restrict__ list,
                                                                                const unsigned int* __restrict__ count,
@@ -171,7 +171,7 @@ size_t staged_state_bytes(int64_t n_rows, int64_t n0) {
   return (size_t)staged_tiles(n_rows, n0) * kStateWords * kNp * kBlock * sizeof(uint64_t);
 }
 
-template <bool MASS>
+template <int MASS>
 cudaError_t launch_staged_m(const rsdev::ShootDesc& d, uint64_t* state, bool first, bool last, int64_t grid,
                             cudaStream_t s) {
   constexpr size_t smem = sizeof(StagedSmem);
@@ -185,8 +185,9 @@ cudaError_t launch_staged(const rsdev::ShootDesc& d, uint64_t* state, bool first
   const int64_t grid = staged_tiles(d.n_rows, d.n0);
   if (grid <= 0) return cudaSuccess;
   if (grid >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
-  return d.f.has_mass ? launch_staged_m<true>(d, state, first, last, grid, s)
-                      : launch_staged_m<false>(d, state, first, last, grid, s);
+  if (d.f.has_mass == rsdev::kWideMass) return launch_staged_m<rsdev::kWideMass>(d, state, first, last, grid, s);
+  return d.f.has_mass ? launch_staged_m<rsdev::kMass>(d, state, first, last, grid, s)
+                      : launch_staged_m<rsdev::kUnitMass>(d, state, first, last, grid, s);
 }
 
 cudaError_t launch_recheck_part(const rsdev::ShootDesc& d, const uint2* list, const unsigned int* count,

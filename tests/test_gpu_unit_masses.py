@@ -8,7 +8,7 @@ import torch
 
 import oracle
 import rs_inputs as ri
-from gpu_helpers import all_rays, dev, rs, shoot_gpu, trace_gpu
+from gpu_helpers import all_rays, dev, per_ray_bound, rs, shoot_gpu, trace_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -101,3 +101,46 @@ def test_streamed_unit_masses_equal_mass_free():
     assert np.array_equal(outs[0][0], outs[1][0]) and outs[0][1] == outs[1][1]
     ref, oref = shoot_gpu(plain)
     assert np.array_equal(outs[1][0], ref) and outs[1][1] == oref
+
+
+@pytest.mark.parametrize("scale", [2.0 ** 60, 2.0 ** 64, 2.0 ** 64 * (1 + 2.0 ** -23), 2.0 ** 100])
+@pytest.mark.parametrize("n", [257, 40])
+def test_masses_about_the_scaled_distance_bound(scale, n):
+    """Largest mass below, at, just above and far above 2^64, where the kernels turn from weighing the distances to
+    weighing 1 / r^2: traces within the float32 bound of the oracle, and the plain, batched, culled and staged maps
+    equal the oracle's.  (60^2 rays: the re-evaluation list holds every ray, as the squared group partials of the
+    error band leave the float32 range here.)"""
+    m = rs()
+    spec = ri.disc_field("wide", n, 0.5, 0.1, 0.2, 60, 40, seed=12, mass="salpeter")
+    spec.masses = (spec.masses / spec.masses.max() * np.float32(1.0)).astype(np.float32)
+    spec.masses = (spec.masses.astype(np.float64) * scale).astype(np.float32)
+    assert float(spec.masses.max()) == np.float32(scale)
+    ij = ri.sample_rays(spec.grid, 400, seed=3)
+    y_ref, _, _ = oracle.trace_field(spec, ij)
+    half = float(np.median(np.abs(y_ref)))
+    spec.window = ri.square_window(half, 40)
+    f = m.Field.from_spec(spec)
+    cut = [0, 256, n] if n > 256 else [0, n]
+    parts = [m.Field(spec.lens_xy[a:b], spec.masses[a:b], spec.kappa_c, spec.gamma) for a, b in zip(cut[:-1], cut[1:])]
+    try:
+        assert f.info() == (n, True)
+        y = f.trace(spec.grid, torch.from_numpy(ij)).cpu().numpy()
+        xy = np.array([[spec.grid.origin[k] + q[k] * spec.grid.spacing[k] for k in (0, 1)] for q in ij])
+        bound = per_ray_bound(spec, xy.astype(np.float32).astype(np.float64), y_ref)
+        assert (np.abs(y - y_ref).max(1) <= bound).all()
+        ref, oref = oracle.shoot_field(spec)
+        maps = [f.shoot(spec.grid, spec.window), f.shoot(spec.grid, spec.window, culled=True)]
+        b = m.Batch([f], [spec.grid], [spec.window])
+        b.launch()
+        maps.append(b.counts[0])
+        c = torch.zeros_like(maps[0])
+        m.rs_shoot_staged([p.handle for p in parts], spec.grid, 0, 60, spec.window, c)
+        maps.append(c)
+        torch.cuda.synchronize()
+        assert f.status() == m.RS_OK
+        for k, c in enumerate(maps):
+            assert np.array_equal(c.cpu().numpy().view(np.uint32), ref), k
+        b.close()
+    finally:
+        for p in [f] + parts:
+            p.close()
