@@ -126,6 +126,75 @@ bool inject_alloc_failure() {
   return false;
 }
 
+constexpr int kPoolDevices = 64;
+struct Pool {
+  cudaMemPool_t pool = nullptr;
+  unsigned long long ctx = 0;  // id of the context the pool belongs to (a device reset ends it)
+  int fields = 0;              // live fields of the device
+};
+static std::mutex g_pool_mutex;
+static Pool g_pools[kPoolDevices];
+
+// Id of the current CUDA context, unique over the process's life (through the driver entry point, so the library
+// needs no link to the driver library); 0 where it cannot be queried.
+static unsigned long long context_id() {
+  using GetId = int (*)(void*, unsigned long long*);
+  static GetId fn = []() -> GetId {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      return nullptr;
+    return reinterpret_cast<GetId>(p);
+  }();
+  unsigned long long id = 0;
+  if (fn == nullptr || fn(nullptr, &id) != 0) return 0;
+  return id;
+}
+
+cudaError_t pool_alloc_async(void** p, size_t bytes, cudaStream_t s) {
+  int dev = -1;
+  cudaMemPool_t pool = nullptr;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kPoolDevices) {
+    const unsigned long long ctx = context_id();
+    std::lock_guard<std::mutex> lock(g_pool_mutex);
+    Pool& q = g_pools[dev];
+    if (ctx != 0 && (q.pool == nullptr || q.ctx != ctx)) {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      uint64_t keep = kPoolKeep;
+      cudaMemPool_t made = nullptr;
+      if (cudaMemPoolCreate(&made, &props) == cudaSuccess &&
+          cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess) {
+        q.pool = made;
+        q.ctx = ctx;
+      } else if (made) {
+        cudaMemPoolDestroy(made);
+      }
+    }
+    if (q.pool != nullptr && q.ctx == ctx) pool = q.pool;
+  }
+  if (pool != nullptr) return cudaMallocFromPoolAsync(p, bytes, pool, s);
+  (void)cudaGetLastError();
+  return cudaMallocAsync(p, bytes, s);  // no pool of our own to be had: the device's default one
+}
+
+void pool_field_created(int device) {
+  if (device < 0 || device >= kPoolDevices) return;
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  ++g_pools[device].fields;
+}
+
+void pool_field_destroyed(int device) {
+  if (device < 0 || device >= kPoolDevices) return;
+  const unsigned long long ctx = context_id();
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  Pool& q = g_pools[device];
+  if (--q.fields == 0 && q.pool != nullptr && q.ctx == ctx) cudaMemPoolTrimTo(q.pool, 0);
+}
+
 int recheck_grid(int device) {
   int v = 0;
   if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || v < 1) v = 1;
@@ -450,6 +519,7 @@ int rs_create_field(const float* lens_xy, const float* masses, int64_t n_lens, d
   f->dev.lamabs = std::nextafter((float)std::max(std::fabs(f->dev.lam1), std::fabs(f->dev.lam2)), INFINITY);
   f->dev.mcap = near_cap(n_lens, f->dev.has_mass ? m_max : 1.f);
   f->dev.status = f->status;
+  pool_field_created(f->device);
   *out = f;
   return RS_OK;
 }
@@ -464,6 +534,7 @@ int rs_destroy_field(rs_field_t f) {
   cudaFree(f->status);
   cudaFree(f->motion);
   if (f->parent) --f->parent->views;
+  pool_field_destroyed(f->device);
   delete f;
   return RS_OK;
 }
@@ -507,6 +578,7 @@ int rs_create_field_view(rs_field_t parent, int64_t lens_begin, int64_t n_lens, 
   f->dev.status = f->status;
   f->parent = parent;
   ++parent->views;
+  pool_field_created(f->device);
   *out = f;
   return RS_OK;
 }
