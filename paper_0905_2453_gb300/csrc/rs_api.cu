@@ -787,8 +787,28 @@ int rs_trace(rs_field_t f, const rs_ray_grid* g, const int64_t* d_ray_ij, int64_
   if (!d_ray_ij || !d_y) return fail(RS_EINVAL, "d_ray_ij / d_y is NULL");
   if (k >= ((int64_t)1 << 31)) return fail(RS_EOVERFLOW, "k must be < 2^31");
   if ((rc = check_field_device(f)) != RS_OK) return rc;
-  cudaError_t e = rsint::launch_trace(f->dev, g->origin[0], g->origin[1], g->spacing[0], g->spacing[1], d_ray_ij, k,
-                                      d_y, d_alpha, d_err, reinterpret_cast<cudaStream_t>(stream));
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  cudaError_t e = cudaSuccess;
+  void* ws = nullptr;
+  if (rsint::trace_split_pays(f->dev.n_lens, k, d_err != nullptr)) {
+    // the split path needs a workspace: without one (or while the stream is being captured, as the call
+    // then leaves no allocation in the graph) the direct kernel gives the same bits
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+        dev_alloc_async(&ws, rsint::trace_split_bytes(f->dev.n_lens, k), s) != cudaSuccess) {
+      ws = nullptr;
+      (void)cudaGetLastError();
+    }
+  }
+  if (ws) {
+    e = rsint::launch_trace_split(f->dev, g->origin[0], g->origin[1], g->spacing[0], g->spacing[1], d_ray_ij, k, d_y,
+                                  d_alpha, d_err, ws, s);
+    const cudaError_t e2 = cudaFreeAsync(ws, s);
+    if (e == cudaSuccess) e = e2;
+  } else {
+    e = rsint::launch_trace(f->dev, g->origin[0], g->origin[1], g->spacing[0], g->spacing[1], d_ray_ij, k, d_y,
+                            d_alpha, d_err, s);
+  }
   if (e != cudaSuccess) return cuda_fail(e, "trace kernel launch");
   return RS_OK;
 }

@@ -428,12 +428,29 @@ __device__ __forceinline__ float ray_coord(int64_t idx, double spacing, double o
 // only underflow when the ray is within ~3e-10 of one of the two lenses, a ray whose own
 // deflection is then ~1e9 (out of any window), and only that ray is affected.
 // ----------------------------------------------------------------------------------------------
-template <bool MONT, int MASS>
+//
+// tr sees every squared distance of ray pair q (NoTrack: nothing; MinTrack: the nearest lens of each ray).
+struct NoTrack {
+  __device__ __forceinline__ void operator()(int, uint64_t) const {}
+};
+struct MinTrack {
+  float* r2;  // smallest squared distance so far of rays 2 q and 2 q + 1
+  __device__ __forceinline__ void operator()(int q, uint64_t v) const {
+    float a, b;
+    f2_unpack(v, a, b);
+    r2[2 * q] = fminf(r2[2 * q], a);
+    r2[2 * q + 1] = fminf(r2[2 * q + 1], b);
+  }
+};
+
+template <bool MONT, int MASS, class TR = NoTrack>
 __device__ __forceinline__ void lens_pair_step(uint64_t d1a, uint64_t d1b, uint64_t E1a, uint64_t E1b, uint64_t E2a,
                                                uint64_t S2a, uint64_t E2b, uint64_t S2b, uint64_t Ma, uint64_t Mb,
-                                               uint64_t& P1, uint64_t& P2) {
+                                               uint64_t& P1, uint64_t& P2, int q = 0, TR tr = TR{}) {
   const uint64_t r2a = f2_fma(d1a, d1a, S2a);
   const uint64_t r2b = f2_fma(d1b, d1b, S2b);
+  tr(q, r2a);
+  tr(q, r2b);
   uint64_t wa, wb;
   if (MONT) {
     const uint64_t pr = f2_mul(r2a, r2b);
@@ -466,10 +483,11 @@ __device__ __forceinline__ uint64_t weigh(uint64_t d, uint64_t M) {
 }
 
 // A single lens (the odd last lens of a field), direct reciprocal.
-template <int MASS>
+template <int MASS, class TR = NoTrack>
 __device__ __forceinline__ void lens_single_step(uint64_t d1, uint64_t E1, uint64_t E2, uint64_t S2, uint64_t M,
-                                                 uint64_t& P1, uint64_t& P2) {
+                                                 uint64_t& P1, uint64_t& P2, int q = 0, TR tr = TR{}) {
   const uint64_t r2 = f2_fma(d1, d1, S2);
+  tr(q, r2);
   float a0, a1;
   f2_unpack(r2, a0, a1);
   uint64_t w = f2_pack(rcp_approx(a0), rcp_approx(a1));
@@ -498,9 +516,10 @@ __device__ __forceinline__ void load_lens(uint32_t lbase, uint32_t mbase, int l,
 
 // One lens pair (lenses l, l + 1) against all ray pairs of the thread, every ray pair with its own
 // x2 (listed rays, cells): d2 and d2^2 are formed per ray pair.
-template <int NP, bool MONT, int MASS>
+template <int NP, bool MONT, int MASS, class TR = NoTrack>
 __device__ __forceinline__ void lens_pair_all(uint32_t lbase, uint32_t mbase, int l, const uint64_t (&X1)[NP],
-                                              const uint64_t (&X2)[NP], uint64_t (&P1)[NP], uint64_t (&P2)[NP]) {
+                                              const uint64_t (&X2)[NP], uint64_t (&P1)[NP], uint64_t (&P2)[NP],
+                                              TR tr = TR{}) {
   uint64_t Lxa, Lya, Ma, Lxb, Lyb, Mb;
   load_lens<MASS>(lbase, mbase, l, Lxa, Lya, Ma);
   load_lens<MASS>(lbase, mbase, l + 1, Lxb, Lyb, Mb);
@@ -510,7 +529,7 @@ __device__ __forceinline__ void lens_pair_all(uint32_t lbase, uint32_t mbase, in
     const uint64_t S2a = f2_mul(D2a, D2a), S2b = f2_mul(D2b, D2b);
     const uint64_t d1a = f2_sub(X1[q], Lxa), d1b = f2_sub(X1[q], Lxb);
     lens_pair_step<MONT, MASS>(d1a, d1b, weigh<MASS>(d1a, Ma), weigh<MASS>(d1b, Mb), weigh<MASS>(D2a, Ma), S2a,
-                               weigh<MASS>(D2b, Mb), S2b, Ma, Mb, P1[q], P2[q]);
+                               weigh<MASS>(D2b, Mb), S2b, Ma, Mb, P1[q], P2[q], q, tr);
   }
 }
 
@@ -558,42 +577,43 @@ struct RayTile {
   static constexpr int WC = R;
 };
 
-template <int RPT, int TILE, bool MONT, int MASS, bool ROW>
+// (tr: only without the row table)
+template <int RPT, int TILE, bool MONT, int MASS, bool ROW, class TR = NoTrack>
 __device__ __forceinline__ void lens_pair_any(uint32_t lbase, uint32_t xbase, uint32_t mbase, uint32_t rt, int l,
                                               const uint64_t (&X1)[RPT / 2], const uint64_t (&X2)[RPT / 2],
-                                              uint64_t (&P1)[RPT / 2], uint64_t (&P2)[RPT / 2]) {
+                                              uint64_t (&P1)[RPT / 2], uint64_t (&P2)[RPT / 2], TR tr = TR{}) {
   if constexpr (ROW)
     lens_pair_rows<RayTile<RPT>::R, RayTile<RPT>::CP, TILE, MONT, MASS>(xbase, mbase, rt, l, X1, P1, P2);
   else
-    lens_pair_all<RPT / 2, MONT, MASS>(lbase, mbase, l, X1, X2, P1, P2);
+    lens_pair_all<RPT / 2, MONT, MASS>(lbase, mbase, l, X1, X2, P1, P2, tr);
 }
 
 // Four lens pairs of a group (lenses l .. l + 7, l a multiple of 8 within the group): the fixed reciprocal pattern.
-template <int RPT, int TILE, int MASS, bool ROW>
+template <int RPT, int TILE, int MASS, bool ROW, class TR = NoTrack>
 __device__ __forceinline__ void lens_block(uint32_t lbase, uint32_t xbase, uint32_t mbase, uint32_t rt, int l,
                                            const uint64_t (&X1)[RPT / 2], const uint64_t (&X2)[RPT / 2],
-                                           uint64_t (&P1)[RPT / 2], uint64_t (&P2)[RPT / 2]) {
-  lens_pair_any<RPT, TILE, mont_pair<MASS>(0), MASS, ROW>(lbase, xbase, mbase, rt, l + 0, X1, X2, P1, P2);
-  lens_pair_any<RPT, TILE, mont_pair<MASS>(1), MASS, ROW>(lbase, xbase, mbase, rt, l + 2, X1, X2, P1, P2);
-  lens_pair_any<RPT, TILE, mont_pair<MASS>(2), MASS, ROW>(lbase, xbase, mbase, rt, l + 4, X1, X2, P1, P2);
-  lens_pair_any<RPT, TILE, mont_pair<MASS>(3), MASS, ROW>(lbase, xbase, mbase, rt, l + 6, X1, X2, P1, P2);
+                                           uint64_t (&P1)[RPT / 2], uint64_t (&P2)[RPT / 2], TR tr = TR{}) {
+  lens_pair_any<RPT, TILE, mont_pair<MASS>(0), MASS, ROW>(lbase, xbase, mbase, rt, l + 0, X1, X2, P1, P2, tr);
+  lens_pair_any<RPT, TILE, mont_pair<MASS>(1), MASS, ROW>(lbase, xbase, mbase, rt, l + 2, X1, X2, P1, P2, tr);
+  lens_pair_any<RPT, TILE, mont_pair<MASS>(2), MASS, ROW>(lbase, xbase, mbase, rt, l + 4, X1, X2, P1, P2, tr);
+  lens_pair_any<RPT, TILE, mont_pair<MASS>(3), MASS, ROW>(lbase, xbase, mbase, rt, l + 6, X1, X2, P1, P2, tr);
 }
 
 // The last, partial group of a field (cnt < 64 lenses from l0): the same pattern by pair index, an odd last
 // lens directly.
-template <int RPT, int TILE, int MASS, bool ROW>
+template <int RPT, int TILE, int MASS, bool ROW, class TR = NoTrack>
 __device__ __forceinline__ void lens_group_partial(uint32_t lbase, uint32_t xbase, uint32_t mbase, uint32_t rt, int l0,
                                                    int cnt, const uint64_t (&X1)[RPT / 2],
                                                    const uint64_t (&X2)[RPT / 2], uint64_t (&P1)[RPT / 2],
-                                                   uint64_t (&P2)[RPT / 2]) {
+                                                   uint64_t (&P2)[RPT / 2], TR tr = TR{}) {
   int p = 0;
   for (; 2 * p + 8 <= cnt; p += 4)  // whole blocks of four pairs first (p = 0 mod 4 at each)
-    lens_block<RPT, TILE, MASS, ROW>(lbase, xbase, mbase, rt, l0 + 2 * p, X1, X2, P1, P2);
+    lens_block<RPT, TILE, MASS, ROW>(lbase, xbase, mbase, rt, l0 + 2 * p, X1, X2, P1, P2, tr);
   for (; 2 * p + 1 < cnt; ++p) {
     if (mont_pair<MASS>(p))
-      lens_pair_any<RPT, TILE, true, MASS, ROW>(lbase, xbase, mbase, rt, l0 + 2 * p, X1, X2, P1, P2);
+      lens_pair_any<RPT, TILE, true, MASS, ROW>(lbase, xbase, mbase, rt, l0 + 2 * p, X1, X2, P1, P2, tr);
     else
-      lens_pair_any<RPT, TILE, false, MASS, ROW>(lbase, xbase, mbase, rt, l0 + 2 * p, X1, X2, P1, P2);
+      lens_pair_any<RPT, TILE, false, MASS, ROW>(lbase, xbase, mbase, rt, l0 + 2 * p, X1, X2, P1, P2, tr);
   }
   if (2 * p < cnt) {
     const int l = l0 + 2 * p;
@@ -615,7 +635,8 @@ __device__ __forceinline__ void lens_group_partial(uint32_t lbase, uint32_t xbas
 #pragma unroll
       for (int q = 0; q < RPT / 2; ++q) {
         const uint64_t D2 = f2_sub(X2[q], Ly), d1 = f2_sub(X1[q], Lx);
-        lens_single_step<MASS>(d1, weigh<MASS>(d1, M), weigh<MASS>(D2, M), f2_mul(D2, D2), M, P1[q], P2[q]);
+        lens_single_step<MASS>(d1, weigh<MASS>(d1, M), weigh<MASS>(D2, M), f2_mul(D2, D2), M, P1[q], P2[q], q,
+                               tr);
       }
     }
   }
@@ -769,6 +790,14 @@ __device__ __forceinline__ bool deflect_accumulate(const FieldDev& f, const uint
   return true;
 }
 
+// Error-band estimate of a ray from its band sums.  |alpha| enters through the rounding of Eq. 6 (~1e-16 |alpha|
+// in float64): 8e-15 (|hi1| + |hi2|).  Every operation is spelled out (here and in band_halfwidth) so that all
+// kernels round alike.
+__device__ __forceinline__ float band_sigma(float ss, float ab, float h1, float h2) {
+  const float eq6 = __fmul_rn(8e-15f, __fadd_rn(fabsf(h1), fabsf(h2)));
+  return __fmaf_rn(kSigmaScale, __fsqrt_rn(ss), __fmaf_rn(kSystematicScale, ab, eq6));
+}
+
 // alpha as float pairs (hi, lo: alpha = hi + lo exactly, |lo| <= ulp(hi) / 2) and the error-band
 // estimate sig of each ray from its accumulators.
 template <int RPT>
@@ -784,10 +813,8 @@ __device__ __forceinline__ void deflect_finish(const DeflectAcc<RPT / 2>& acc, f
     float s, sB, b, bB;
     f2_unpack(acc.SS[q], s, sB);
     f2_unpack(acc.AB[q], b, bB);
-    // |alpha| enters through the rounding of Eq. 6 (~1e-16 |alpha| in float64): 8e-15 (|hi1| + |hi2|)
-    sig[2 * q] = kSigmaScale * sqrtf(s) + kSystematicScale * b + 8e-15f * (fabsf(a1h[2 * q]) + fabsf(a2h[2 * q]));
-    sig[2 * q + 1] =
-        kSigmaScale * sqrtf(sB) + kSystematicScale * bB + 8e-15f * (fabsf(a1h[2 * q + 1]) + fabsf(a2h[2 * q + 1]));
+    sig[2 * q] = band_sigma(s, b, a1h[2 * q], a2h[2 * q]);
+    sig[2 * q + 1] = band_sigma(sB, bB, a1h[2 * q + 1], a2h[2 * q + 1]);
   }
 }
 
@@ -852,7 +879,8 @@ __device__ __forceinline__ bool deflect(const FieldDev& f, const float (&x1)[RPT
 // evaluation of Eq. 6), the near-lens term of the ray's largest-term bound tn, and the lam x part of
 // the Eq. 6 rounding.  The shoot's float-float epilogue adds its own rounding bound on top (ff_pixel).
 __device__ __forceinline__ float band_halfwidth(float sig, float tn, float lamabs, float x1, float x2) {
-  return sig + kNearScale * tn + 4e-15f * lamabs * (fabsf(x1) + fabsf(x2));
+  const float eq6 = __fmul_rn(__fmul_rn(4e-15f, lamabs), __fadd_rn(fabsf(x1), fabsf(x2)));
+  return __fadd_rn(__fmaf_rn(kNearScale, tn, sig), eq6);
 }
 
 // ----------------------------------------------------------------------------------------------

@@ -81,6 +81,20 @@ cudaError_t shoot_blocks_per_sm(int cfg, bool mass, int* blocks);
 cudaError_t launch_trace(const rsdev::FieldDev& f, double or0, double or1, double sp0, double sp1,
                          const int64_t* ij, int64_t k, double* y, double* alpha, double* err, cudaStream_t s);
 
+// The same with the lens groups of every ray summed side by side (rs_trace.cu): ws holds trace_split_bytes, which
+// the workspace bound kTraceSplitBytes keeps below 32 MiB + 36 bytes per ray.  It pays where the direct kernel
+// (one thread per four rays over all lenses) leaves SMs idle or runs long serial loops; measured alone, us,
+// direct / split without | with error bands: 512 lenses x 1000 rays 54 / 67 | 115 / 82, 2000 x 4096 95 / 75 |
+// 318 / 84, 2000 x 65536 96 / 108 | 323 / 168, 20000 x 30000 596 / 300 | 4828 / 475, 1e6 x 10 27475 / 915.
+constexpr size_t kTraceSplitBytes = (size_t)32 << 20;
+inline bool trace_split_pays(int n_lens, int64_t k, bool err) {
+  return err ? n_lens >= 512 && k <= 65536 : n_lens >= 1024 && k <= 32768;
+}
+size_t trace_split_bytes(int n_lens, int64_t k);
+cudaError_t launch_trace_split(const rsdev::FieldDev& f, double or0, double or1, double sp0, double sp1,
+                               const int64_t* ij, int64_t k, double* y, double* alpha, double* err, void* ws,
+                               cudaStream_t s);
+
 // Listed rays -> source positions in float-float (the certified re-evaluation).
 cudaError_t launch_trace_ff(const rsdev::FieldDev& f, double or0, double or1, double sp0, double sp1,
                             const int64_t* ij, int64_t k, double* y, double* alpha, cudaStream_t s);
