@@ -357,7 +357,9 @@ int rs_field_status(rs_field_t f, int clear, int* status);
  * rs_set_launch_config selects the shape used by rs_shoot / rs_shoot_rows /
  * rs_shoot_rows_noalloc (and by batches planned afterwards) for fields without
  * (has_masses = 0) or with per-lens masses; RS_EINVAL for a shape that is not
- * compiled.  rs_launch_configs lists the compiled shapes: up to `cap`
+ * compiled.  Until it is called for a mass mode the library takes a shape per call by the
+ * number of lenses and rays (batches: by the number of lenses of each field), and
+ * rs_get_launch_config reports 128 x 8 x 512 at two CTAs per SM.  rs_launch_configs lists the compiled shapes: up to `cap`
  * (block, rpt, lens_tile, min_ctas) quadruples into `shapes` (int[4*cap]);
  * returns the number available via *count.  rs_launch_occupancy reports how
  * many CTAs of a shape's shoot kernel are resident per SM on the current device

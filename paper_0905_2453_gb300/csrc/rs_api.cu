@@ -108,8 +108,9 @@ __global__ void selftest_wait_kernel(uint64_t limit_ns, unsigned int* out) {
 namespace rshost {
 
 thread_local std::string g_err;
-// Launch shape per mass mode (index 0: unit masses, 1: per-lens masses).
+// Launch shape per mass mode (index 0: unit masses, 1: per-lens masses), and whether the caller set it.
 int g_cfg[2] = {rsint::kDefaultCfg, rsint::kDefaultCfg};
+bool g_cfg_set[2] = {false, false};
 // Certified binning (float-float re-evaluation of rays inside their error band of a pixel edge).
 int g_certify = 1;
 // Device memory for the per-ray state of a staged (lens-partitioned) shoot; larger calls run in row blocks.
@@ -316,6 +317,25 @@ float near_cap(int64_t n_lens, float m_max) {
   return n_lens > 0 ? m_max : 0.f;
 }
 
+// Measured on squares of 256^2 to 4096^2 rays, 100 to 60000 lenses, unit and Salpeter masses, us (128x8x512 at two
+// CTAs per SM / the shape taken):
+//   * few lenses: a CTA's start and its per-ray epilogue weigh more than its sums, and sixteen warps per SM hide
+//     them: 128x4x256 at four CTAs per SM (100 lenses x 1000^2: 60.3 / 50.9, x 4096^2: 746 / 553; 300 x 1000^2:
+//     102 / 87; at 1000 lenses level: 3078 / 3100 for 4096^2).
+//   * fewer than one small CTA per SM: the largest share of an SM decides, four rays per thread (300 x 256^2: 31.7 /
+//     23.6, 60000 x 256^2: 2215 / 1369).
+//   * else 128x8x512 at three CTAs per SM (1e4 x 1536^2: 4375 / 4316; Salpeter 3000 x 4096^2: 9625 / 9240; nowhere
+//     more than 2 % behind).
+int pick_cfg(const rs_field* f, int64_t n_rows, int64_t n0) {
+  const int mass = f->dev.has_mass != rsdev::kUnitMass ? 1 : 0;
+  if (g_cfg_set[mass]) return g_cfg[mass];
+  constexpr int64_t kFewLenses = 768;
+  // CTAs of four warps x four rays per thread
+  const int64_t small = ((n_rows + 3) / 4) * ((n0 + 127) / 128);
+  if (f->n_lens > 256 && small <= num_sms(f->device)) return rsint::kFewRaysCfg;
+  return f->n_lens < kFewLenses ? rsint::kFewLensesCfg : rsint::kManyLensesCfg;
+}
+
 int mass_mode(bool weighted, float m_max) {
   if (!weighted) return rsdev::kUnitMass;
   return m_max <= rsdev::kMassMax ? rsdev::kMass : rsdev::kWideMass;  // NaN (device inputs): the wide kernels
@@ -352,6 +372,7 @@ int rs_set_launch_config(int has_masses, int block, int rays_per_thread, int len
     return fail(RS_EINVAL, "no compiled launch shape (%d threads, %d rays/thread, %d-lens tiles, %d CTAs/SM)", block,
                 rays_per_thread, lens_tile, min_ctas);
   g_cfg[has_masses ? 1 : 0] = c;
+  g_cfg_set[has_masses ? 1 : 0] = true;
   return RS_OK;
 }
 
@@ -713,7 +734,7 @@ int rs_shoot_rows(rs_field_t f, const rs_ray_grid* g, int64_t row_begin, int64_t
     d.rc_list = reinterpret_cast<uint2*>(reinterpret_cast<char*>(ws) + 16);
     e = cudaMemsetAsync(d.rc_count, 0, sizeof(unsigned int), s);
   }
-  if (e == cudaSuccess) e = rsint::launch_shoot(g_cfg[f->dev.has_mass ? 1 : 0], d, s);
+  if (e == cudaSuccess) e = rsint::launch_shoot(pick_cfg(f, d.n_rows, d.n0), d, s);
   if (e == cudaSuccess && ws) e = rsint::launch_recheck(&d, nullptr, d.rc_list, d.rc_count, d.rc_cap, recheck_grid(f->device), s);
   if (ws) {
     cudaError_t e2 = cudaFreeAsync(ws, s);
@@ -970,7 +991,7 @@ extern "C" int rs_shoot_rows_noalloc(rs_field_t f, const rs_ray_grid* g, int64_t
   d.rc_cap = cap;
   // the array keeps the previous call's contents: only the counter must start at zero
   cudaError_t e = cudaMemsetAsync(d.rc_count, 0, sizeof(unsigned int), s);
-  if (e == cudaSuccess) e = rsint::launch_shoot(g_cfg[f->dev.has_mass ? 1 : 0], d, s);
+  if (e == cudaSuccess) e = rsint::launch_shoot(pick_cfg(f, d.n_rows, d.n0), d, s);
   if (e == cudaSuccess) e = rsint::launch_recheck(&d, nullptr, d.rc_list, d.rc_count, d.rc_cap, recheck_grid(f->device), s);
   if (e != cudaSuccess) return cuda_fail(e, "shoot launch (no-allocation variant)");
   return RS_OK;

@@ -64,7 +64,8 @@ int rs_batch_create_shaped(int n_fields, const rs_field_t* fields, const rs_ray_
                         d_out_of_window ? d_out_of_window + k : nullptr, &descs[k])) != RS_OK)
       return rc;
     const int mass = fields[k]->dev.has_mass;
-    int cfg = g_cfg[mass ? 1 : 0];
+    // without a shape of the caller's: by lens count only, as the other fields fill the chip
+    int cfg = pick_cfg(fields[k], (int64_t)1 << 20, (int64_t)1 << 10);
     if (shapes) {
       const int* sh = shapes + 4 * k;
       cfg = rsint::find_cfg(sh[0], sh[1], sh[2], sh[3]);
@@ -164,15 +165,40 @@ int rs_batch_create_shaped(int n_fields, const rs_field_t* fields, const rs_ray_
     for (int grp = 0; grp < G; ++grp)
       if (b->n_items[grp] > 0) order.push_back(grp);
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return items[x][0].cost > items[y][0].cost; });
+    // the groups are independent: one branch of the graph each, so that a group's CTAs start where another
+    // group's last ones leave SMs idle
+    std::vector<cudaStream_t> side(order.size(), nullptr);
+    std::vector<cudaEvent_t> done(order.size(), nullptr);
+    cudaEvent_t fork = nullptr;
+    if (e == cudaSuccess && order.size() > 1) {
+      e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+      if (e == cudaSuccess) e = cudaEventRecord(fork, cs);
+    }
     for (size_t i = 0; i < order.size() && e == cudaSuccess; ++i) {
       const int grp = order[i];
-      e = rsint::launch_batch(grp / rs_batch::kMassModes, grp % rs_batch::kMassModes, b->d_descs, b->d_items + b->item_offset[grp], b->n_items[grp],
-                              b->d_counter + grp, b->grid[grp], cs);
+      cudaStream_t bs = cs;
+      if (i > 0) {
+        e = cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done[i], cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(side[i], fork, 0);
+        bs = side[i];
+      }
+      if (e == cudaSuccess)
+        e = rsint::launch_batch(grp / rs_batch::kMassModes, grp % rs_batch::kMassModes, b->d_descs,
+                                b->d_items + b->item_offset[grp], b->n_items[grp], b->d_counter + grp, b->grid[grp],
+                                bs);
+      if (e == cudaSuccess && i > 0) e = cudaEventRecord(done[i], bs);
     }
+    for (size_t i = 1; i < order.size() && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(cs, done[i], 0);
     if (e == cudaSuccess && b->rc_cap > 0)
       e = rsint::launch_recheck(nullptr, b->d_descs, b->d_rc_list, b->d_rc_count, b->rc_cap, recheck_grid(dev), cs);
     cudaError_t e2 = cudaStreamEndCapture(cs, &b->graph);
     if (e == cudaSuccess) e = e2;
+    for (size_t i = 1; i < order.size(); ++i) {
+      if (done[i]) cudaEventDestroy(done[i]);
+      if (side[i]) cudaStreamDestroy(side[i]);
+    }
+    if (fork) cudaEventDestroy(fork);
   }
   if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
   cudaStreamDestroy(cs);

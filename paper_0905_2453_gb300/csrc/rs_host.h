@@ -32,6 +32,8 @@ namespace rshost {
 
 // Launch shape per mass mode (index 0: unit masses, 1: per-lens masses).
 extern int g_cfg[2];
+// Shape of a call of n_rows x n0 rays through f: the caller's (rs_set_launch_config), or by size.
+int pick_cfg(const rs_field* f, int64_t n_rows, int64_t n0);
 // Certified binning (float-float re-evaluation of rays inside their error band of a pixel edge).
 extern int g_certify;
 // Device memory for the per-ray state of a staged (lens-partitioned) shoot; larger calls run in row blocks.
