@@ -3,15 +3,19 @@
 // shows that none of its rays can land in the window, and the others are shot with the same per-ray
 // arithmetic as rs_shoot, so the counts and the out-of-window count equal those of rs_shoot.
 //
-// Bound for a cell with ray box centre c and circumradius rho (every ray x of the cell has
-// |x - c| <= rho), lenses at distance d_i = |c - x_i| > rho:
-//   |alpha(x) - alpha(c)| <= sum_i m_i |x - c| / (|x - x_i| |c - x_i|) <= rho sum_i m_i / (d_i (d_i - rho)) = B
-// (from |a/|a|^2 - b/|b|^2| = |a - b| / (|a| |b|)), and sum_i m_i / |x - x_i| <= sum_i m_i / (d_i - rho) = S,
-// which bounds the float32 error band of every ray of the cell (a small multiple of 2^-24 S).  So
-// y_k(x) = lam_k x_k - alpha_k(x) lies within [min, max](lam_k x_k) - alpha_k(c) +- (B + margins); a cell
-// whose box misses the window on some axis is skipped and its rays are counted out of window.  A
-// cell with a lens within 1.02 rho of c has no finite bound and is always shot.  The bound is applied
-// to cells of 64 x 64 rays first and then to the 16 x 16 cells of the kept ones.
+// Bound for a cell with ray box centre c and circumradius rho (every ray x = c + h of the cell has |h| <= rho),
+// lenses at distance d_i = |c - x_i| > rho.  In complex notation conj(alpha(z)) = f(z) = sum_i m_i / (z - z_i), and
+// 1 / (w + h) = 1 / w - h / w^2 + h^2 / (w^2 (w + h)) with w = c - z_i gives
+//   |f(c + h) - f(c) - f'(c) h| <= rho^2 sum_i m_i / (d_i^2 (d_i - rho)) = rho^2 B,    f'(c) = -sum_i m_i / w_i^2.
+// So with q1 = sum_i m_i (dx^2 - dy^2) / d^4, q2 = sum_i 2 m_i dx dy / d^4 the cell's source positions are
+//   y1 = lam1 c1 - alpha1(c) + (lam1 + q1) h1 + q2 h2 +- rho^2 B,   y2 = lam2 c2 - alpha2(c) + q2 h1 + (lam2 - q1) h2 +- rho^2 B,
+// and sum_i m_i / |x - x_i| <= sum_i m_i / (d_i - rho) = S bounds the rounding of every ray of the cell.  A cell
+// whose box misses the window on some axis is skipped and its rays are counted out of window.  A cell with a lens
+// within 1.02 rho of c has no finite bound and is always shot.  The bound is applied to cells of 64 x 64 rays first
+// and then to the 16 x 16 cells of the kept ones.
+//
+// The linear term is what makes the bound worth its cost: without it (|alpha(x) - alpha(c)| <= rho sum m / (d (d -
+// rho))) the x4 zoom of the 1e4-lens map shot 8.52e6 rays for 4.12e6 in the window.
 #include "rs_internal.h"
 
 namespace {
@@ -83,6 +87,7 @@ __global__ void __launch_bounds__(kCullBlock)
   const float rho = (float)(sqrt(h1 * h1 + h2 * h2) * (1.0 + 0x1p-20)) + 1e-30f;
   const float rho_near = 1.02f * rho;  // d <= 1.02 rho: no usable bound
   float a1h = 0.f, a1l = 0.f, a2h = 0.f, a2l = 0.f, bh = 0.f, bl = 0.f, sh = 0.f, sl = 0.f;
+  float q1h = 0.f, q1l = 0.f, q2h = 0.f, q2l = 0.f;
   bool near = false;
   const int n = d.f.n_lens;
   for (int t0 = 0; t0 < n; t0 += kCullBlock) {
@@ -95,7 +100,7 @@ __global__ void __launch_bounds__(kCullBlock)
     __syncthreads();
     const int cnt = min(kCullBlock, n - t0);
     for (int g = 0; g < cnt; g += 32) {
-      float pa1 = 0.f, pa2 = 0.f, pb = 0.f, ps = 0.f;
+      float pa1 = 0.f, pa2 = 0.f, pb = 0.f, ps = 0.f, pq1 = 0.f, pq2 = 0.f;
       const int ge = min(g + 32, cnt);
       for (int q = g; q < ge; ++q) {
         const float4 L = s_lens[q];
@@ -105,15 +110,21 @@ __global__ void __launch_bounds__(kCullBlock)
         const float rs = rsqrt_approx(d2);
         const float dist = d2 * rs;
         near |= !(dist > rho_near);  // NaN (a lens on the centre) counts as near
-        const float mi = m * rs * rs;
+        const float r2 = rs * rs;
+        const float mi = m * r2;
         pa1 = fmaf(mi, dx, pa1);
         pa2 = fmaf(mi, dy, pa2);
+        const float mq = mi * r2;
+        pq1 = fmaf(mq, fmaf(dx, dx, -(dy * dy)), pq1);
+        pq2 = fmaf(mq, dx * dy, pq2);
         const float mg = m * rcp_approx(dist - rho);
         ps += mg;
-        pb = fmaf(mg, rs, pb);
+        pb = fmaf(mg, r2, pb);
       }
       fold(a1h, a1l, pa1);
       fold(a2h, a2l, pa2);
+      fold(q1h, q1l, pq1);
+      fold(q2h, q2l, pq2);
       fold(bh, bl, pb);
       fold(sh, sl, ps);
     }
@@ -123,22 +134,24 @@ __global__ void __launch_bounds__(kCullBlock)
   bool keep = true;
   if (!near) {
     // terms carry a few 2^-22 relative (approximate reciprocal square root and reciprocal, the gap's
-    // cancellation when d is near 1.02 rho: <= 2^-16), sums of 32 float terms ~2^-19 of their
+    // cancellation when d is near 1.02 rho: <= 2^-15), sums of 32 float terms ~2^-19 of their
     // absolute sum: inflate B and S by 2^-8
     const double S = ((double)sh + (double)sl) * (1.0 + 0x1p-8);
-    const double B = (double)rho * ((double)bh + (double)bl) * (1.0 + 0x1p-8);
+    const double B = (double)rho * (double)rho * ((double)bh + (double)bl) * (1.0 + 0x1p-8);
     const double A1 = (double)a1h + (double)a1l, A2 = (double)a2h + (double)a2l;
-    // alpha(c) error <= ~2^-18 S; the float32 band of a ray <= ~59 u S(x) <= 2^-18 S; float64 roundings
+    const double Q1 = (double)q1h + (double)q1l, Q2 = 2.0 * ((double)q2h + (double)q2l);
+    // alpha(c) error <= ~2^-18.4 S, a ray's float32 error <= 72 u S = 2^-17.8 S, the linear term's error <= rho 2^-18
+    // sum m / d^2 <= 2^-20 S per coefficient (rho (d - rho) <= d^2 / 4): together below 2^-16 S, taken twice; and
+    // float64 roundings
     const double x1m = fmax(fabs((double)xa1), fabs((double)xb1)), x2m = fmax(fabs((double)xa2), fabs((double)xb2));
-    const double M = B + 0x1p-11 * S +
+    const double M = B + 0x1p-15 * S +
                      0x1p-40 * (fabs(d.f.lam1) * x1m + fabs(d.f.lam2) * x2m + fabs(A1) + fabs(A2) + B + 1.0 +
                                 fabs(d.lo0) + fabs(d.lo1) + fabs(hi0) + fabs(hi1));
-    const double p1 = d.f.lam1 * (double)xa1, q1 = d.f.lam1 * (double)xb1;
-    const double p2 = d.f.lam2 * (double)xa2, q2 = d.f.lam2 * (double)xb2;
-    const double y1min = fmin(p1, q1) - A1 - M, y1max = fmax(p1, q1) - A1 + M;
-    const double y2min = fmin(p2, q2) - A2 - M, y2max = fmax(p2, q2) - A2 + M;
-    const bool finite = isfinite(M) && isfinite(A1) && isfinite(A2);
-    keep = !finite || !(y1max < d.lo0 || y1min > hi0 || y2max < d.lo1 || y2min > hi1);
+    const double y1 = d.f.lam1 * (double)c1 - A1, y2 = d.f.lam2 * (double)c2 - A2;
+    const double e1 = (fabs(d.f.lam1 + Q1) * h1 + fabs(Q2) * h2) * (1.0 + 0x1p-40) + M;
+    const double e2 = (fabs(Q2) * h1 + fabs(d.f.lam2 - Q1) * h2) * (1.0 + 0x1p-40) + M;
+    const bool finite = isfinite(e1) && isfinite(e2) && isfinite(A1) && isfinite(A2);
+    keep = !finite || !(y1 + e1 < d.lo0 || y1 - e1 > hi0 || y2 + e2 < d.lo1 || y2 - e2 > hi1);
   }
   if (keep) {
     const unsigned slot = atomicAdd(out_count, 1u);
