@@ -16,7 +16,7 @@ struct rs_lc_plan {
   int profile;
   double cut2;
   float ecut;
-  int grid;
+  int parts;
   rsint::LcTrack* d_table;
 };
 
@@ -105,8 +105,9 @@ int lc_prepare(int n_maps, const float* const* d_mu, const rs_window* windows, i
     if (!(d.a0 > 0.f && d.a1 > 0.f && std::isfinite(d.a0) && std::isfinite(d.a1) && std::isfinite(d.inv_a0)))
       return fail(RS_EINVAL, "map %d: pixel / profile size ratio outside the float32 range", tr.map);
     // the float32 exponent is within ~8u ((R + pix0)^2 + (R + pix1)^2) escale + 4u E of the exact one
-    // (offsets in pixel units carry u (|offset| + 1)); the band takes 2^-16 of that scale (~30x margin)
-    d.band = (float)(std::ldexp((std::pow(R + pix[0], 2) + std::pow(R + pix[1], 2)) * escale + ecut_d, -16));
+    // (offsets in pixel units carry u (|offset| + 1)); the band takes 2^-18 of that scale (8x margin: wider
+    // bands send more pixels, and with them whole warps, through the tests)
+    d.band = (float)(std::ldexp((std::pow(R + pix[0], 2) + std::pow(R + pix[1], 2)) * escale + ecut_d, -18));
     d.n = tr.n;
     d.out_off = off;
     off += tr.n;
@@ -117,9 +118,10 @@ int lc_prepare(int n_maps, const float* const* d_mu, const rs_window* windows, i
   return RS_OK;
 }
 
-int lc_grid(int device, int64_t total) {
-  const int64_t want = (total + 255) / 256;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms(device) * 8));
+int lc_row_parts(const LcPlan& p, int device) {
+  double rows = 0.0;
+  for (const rsint::LcTrack& t : p.table) rows = std::max(rows, 2.0 * t.rp1);
+  return rsint::lc_parts(num_sms(device), p.total, rows);
 }
 
 }  // namespace
@@ -145,7 +147,7 @@ int rs_light_curves(int n_maps, const float* const* d_mu, const rs_window* windo
   e = cudaMemcpyAsync(d_table, plan.table.data(), bytes, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = rsint::launch_light_curves(plan.profile, d_table, (int)plan.table.size(), plan.total, plan.cut2, plan.ecut,
-                                   d_mu_out, d_dm_out, lc_grid(dev, plan.total), st);
+                                   d_mu_out, d_dm_out, lc_row_parts(plan, dev), st);
   cudaFreeAsync(d_table, st);
   if (e != cudaSuccess) return cuda_fail(e, "light-curve kernel");
   return RS_OK;
@@ -170,7 +172,7 @@ int rs_light_curve_plan_create(int n_maps, const float* const* d_mu, const rs_wi
   p->profile = plan.profile;
   p->cut2 = plan.cut2;
   p->ecut = plan.ecut;
-  p->grid = lc_grid(p->device, plan.total);
+  p->parts = lc_row_parts(plan, p->device);
   if (p->n_tracks > 0) {
     const size_t bytes = plan.table.size() * sizeof(rsint::LcTrack);
     if ((e = dev_alloc(&p->d_table, bytes)) != cudaSuccess) {
@@ -202,7 +204,7 @@ int rs_light_curve_plan_launch(rs_lc_plan_t p, double* d_mu_out, double* d_dm_ou
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
   if (cur != p->device) return fail(RS_EINVAL, "plan lives on device %d but device %d is current", p->device, cur);
   e = rsint::launch_light_curves(p->profile, p->d_table, p->n_tracks, p->total, p->cut2, p->ecut, d_mu_out, d_dm_out,
-                                 p->grid, reinterpret_cast<cudaStream_t>(stream));
+                                 p->parts, reinterpret_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "light-curve kernel");
   return RS_OK;
 }

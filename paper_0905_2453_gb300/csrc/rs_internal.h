@@ -167,7 +167,10 @@ struct LcTrack {
 };
 
 // profile: 0 Gaussian, 1 disc.  cut2: the float64 squared support radius; ecut: the cut in exponent units.
+// parts: warps that share a sample's rows (lc_parts: more than one where one thread per sample would leave SMs
+// short of warps and the largest support of the tracks, max_rows rows, gives each part four rows or more).
+int lc_parts(int sms, int64_t n_samples, double max_rows);
 cudaError_t launch_light_curves(int profile, const LcTrack* tracks, int n_tracks, int64_t n_samples, double cut2,
-                                float ecut, double* mu_out, double* dm_out, int grid, cudaStream_t s);
+                                float ecut, double* mu_out, double* dm_out, int parts, cudaStream_t s);
 
 }  // namespace rsint

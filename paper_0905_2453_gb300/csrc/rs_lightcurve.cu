@@ -1,9 +1,9 @@
 // Light curves of magnification maps (Section 1): the profile-weighted mean of a map around each
 // sample of a straight source track, and its magnitude change -2.5 log10 mu.
 //
-// One thread per sample; the 32 samples of a warp are consecutive samples of (mostly) one track,
-// so the warp's loads of neighbouring pixels fall in the same L1 lines and every per-sample
-// float64 step (position, box, quotient) is paid once per thread, not once per pixel.  A thread
+// One thread per sample (or several, a share of its rows each); the 32 samples of a warp are consecutive samples
+// of (mostly) one track, so the warp's loads of neighbouring pixels fall in the same L1 lines and every per-sample
+// float64 step (position, box, quotient) is paid once per sample, not once per pixel.  A thread
 // walks the rows of the box that bounds its profile's support and, per row, the chord of the
 // support (a margin of ~2^-10 pixel each side).  With E = (di)^2 a0 + (dj)^2 a1 the float32 exponent of
 // the pixel offset (di, dj) in pixel units, the chord's interior (E below the cut by more than a
@@ -14,6 +14,8 @@
 // Gaussian weights are 2^-E with the exponent pre-scaled by log2(e) (one MUFU ex2).  Each row's
 // partial sums are plain float32 (at most 2 R / pix + 3 terms); the rows are folded into compensated
 // (TwoSum) float32 pairs and the mean is their float-float quotient.
+#include <algorithm>
+
 #include "rs_internal.h"
 
 namespace {
@@ -65,74 +67,134 @@ __device__ __forceinline__ void rim_pixel(const LcTrack& T, int64_t k, int i, in
   }
 }
 
-// Gaussian weights are separable: 2^-(ex + ey) = 2^-ex 2^-ey.  A thread whose support box spans at most
-// kLcCols columns keeps the column factors 2^-ex of its sample in shared memory (thread-private slots,
-// conflict-free: slot c of thread t at c * 256 + t) and the untested chord interiors cost a load and a
-// fused multiply-add per pixel; each row's interior sums are scaled by 2^-ey once.
+// Gaussian weights are separable: 2^-(ex + ey) = 2^-ex 2^-ey.  Where a sample's support box spans at most
+// kLcCols columns its column factors 2^-ex are kept in shared memory (slot c of sample s at c * samples + s:
+// conflict-free) and the untested chord interiors cost a load and a fused multiply-add per pixel; each row's
+// interior sums are scaled by 2^-ey once.
 constexpr int kLcThreads = 256;
 constexpr int kLcCols = 32;
 
-template <int PROFILE>
+// A sample as its row parts need it.
+struct LcSample {
+  int track;     // -1: no sample here, or its box misses the map
+  int it, jt;    // floor of the position in pixel units
+  float fx, fy;  // and its fraction
+};
+
+// L warps share 32 samples, warp p of them taking every L-th row of the support from row p on: the 32 lanes of a
+// warp stay consecutive samples whose loads fall in the same L1 lines, the float64 set-up of a sample is done
+// once, and a call of few samples with large supports still fills the chip (L = 1: one thread per sample).
+template <int PROFILE, int L>
 __global__ void __launch_bounds__(kLcThreads) light_curve_kernel(const LcTrack* __restrict__ tracks, int n_tracks,
                                                                  int64_t n_samples, double cut2, float ecut,
                                                                  double* __restrict__ mu_out,
                                                                  double* __restrict__ dm_out) {
-  __shared__ float s_wx[PROFILE == 0 ? kLcCols * kLcThreads : 1];
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n_samples; g += stride) {
-    // the track holding sample g: the last one whose first output position is <= g
-    int lo = 0, hi = n_tracks - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (tracks[mid].out_off <= g) lo = mid; else hi = mid - 1;
-    }
-    const LcTrack& T = tracks[lo];
-    const int64_t k = g - T.out_off;
-    // sample position in pixel-index units (pixel i has its centre at t = i)
-    const double t0 = fma((double)k, T.d0, T.t00);
-    const double t1 = fma((double)k, T.d1, T.t01);
-    float sw = 0.f, cw = 0.f, sm = 0.f, cm = 0.f;
-    if (t0 > -T.rp0 - 2.0 && t0 < (double)T.np0 + T.rp0 + 1.0 && t1 > -T.rp1 - 2.0 &&
-        t1 < (double)T.np1 + T.rp1 + 1.0) {
-      const double ti = floor(t0), tj = floor(t1);
-      const int it = (int)ti, jt = (int)tj;
-      const float fx = (float)(t0 - ti), fy = (float)(t1 - tj);
-      const float rpx = (float)T.rp0, rpy = (float)T.rp1;
-      const int i_lo = max(it + (int)ceilf(fx - rpx) - 1, 0), i_hi = min(it + (int)floorf(fx + rpx) + 1, T.np0 - 1);
-      const int j_lo = max(jt + (int)ceilf(fy - rpy) - 1, 0), j_hi = min(jt + (int)floorf(fy + rpy) + 1, T.np1 - 1);
-      const float a0 = T.a0, a1 = T.a1, band = T.band;
-      const float lim_hi = ecut + band, lim_lo = ecut - band;
-      const bool sep = PROFILE == 0 && i_hi - i_lo < kLcCols;
-      if (sep) {
-        for (int i = i_lo; i <= i_hi; ++i) {
-          const float dxp = __fsub_rn((float)(i - it), fx);
-          s_wx[(i - i_lo) * kLcThreads + threadIdx.x] = ex2_neg(__fmul_rn(__fmul_rn(dxp, dxp), a0));
+  constexpr int S = kLcThreads / L;  // samples of a CTA
+  __shared__ float s_wx[PROFILE == 0 ? kLcCols * S : 1];
+  __shared__ LcSample s_sample[L > 1 ? S : 1];
+  __shared__ float4 s_part[L > 1 ? kLcThreads : 1];  // {sw, cw, sm, cm} of every part
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int part = warp % L, sid = warp / L * 32 + lane;
+  const int64_t stride = (int64_t)gridDim.x * S;
+  for (int64_t base = (int64_t)blockIdx.x * S; base < n_samples; base += stride) {  // CTA-uniform
+    const int64_t g = base + sid;
+    LcSample me;
+    if (part == 0) {
+      me.track = -1;
+      me.it = me.jt = 0;
+      me.fx = me.fy = 0.f;
+      if (g < n_samples) {
+        // the track holding sample g: the last one whose first output position is <= g
+        int lo = 0, hi = n_tracks - 1;
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (tracks[mid].out_off <= g) lo = mid; else hi = mid - 1;
+        }
+        const LcTrack& T = tracks[lo];
+        const int64_t k = g - T.out_off;
+        // sample position in pixel-index units (pixel i has its centre at t = i)
+        const double t0 = fma((double)k, T.d0, T.t00);
+        const double t1 = fma((double)k, T.d1, T.t01);
+        if (t0 > -T.rp0 - 2.0 && t0 < (double)T.np0 + T.rp0 + 1.0 && t1 > -T.rp1 - 2.0 &&
+            t1 < (double)T.np1 + T.rp1 + 1.0) {
+          const double ti = floor(t0), tj = floor(t1);
+          me.track = lo;
+          me.it = (int)ti;
+          me.jt = (int)tj;
+          me.fx = (float)(t0 - ti);
+          me.fy = (float)(t1 - tj);
         }
       }
-      for (int j = j_lo; j <= j_hi; ++j) {
+      if (L > 1) s_sample[sid] = me;
+    }
+    if (L > 1) {
+      __syncthreads();
+      if (part != 0) me = s_sample[sid];
+    }
+    float sw = 0.f, cw = 0.f, sm = 0.f, cm = 0.f;
+    const bool live = me.track >= 0;
+    const LcTrack& T = tracks[live ? me.track : 0];
+    const int64_t k = g - T.out_off;
+    const int it = me.it, jt = me.jt;
+    const float fx = me.fx, fy = me.fy;
+    const float rpx = (float)T.rp0, rpy = (float)T.rp1;
+    const int i_lo = max(it + (int)ceilf(fx - rpx) - 1, 0), i_hi = min(it + (int)floorf(fx + rpx) + 1, T.np0 - 1);
+    const int j_lo = max(jt + (int)ceilf(fy - rpy) - 1, 0), j_hi = min(jt + (int)floorf(fy + rpy) + 1, T.np1 - 1);
+    const float a0 = T.a0, a1 = T.a1, band = T.band, inv_a0 = T.inv_a0;
+    const bool sep = PROFILE == 0 && i_hi - i_lo < kLcCols;
+    if (sep && live) {
+      for (int i = i_lo + part; i <= i_hi; i += L) {
+        const float dxp = __fsub_rn((float)(i - it), fx);
+        s_wx[(i - i_lo) * S + sid] = ex2_neg(__fmul_rn(__fmul_rn(dxp, dxp), a0));
+      }
+    }
+    if (L > 1) __syncthreads();
+    if (live) {
+      const float lim_hi = ecut + band, lim_lo = ecut - band;
+      const float delta = band * inv_a0;  // the guard band in squared pixels of axis 0
+      for (int j = j_lo + part; j <= j_hi; j += L) {
         const float dyp = __fsub_rn((float)(j - jt), fy);
         const float ey = __fmul_rn(__fmul_rn(dyp, dyp), a1);
         const float rem_hi = lim_hi - ey;
         if (!(rem_hi >= 0.f)) continue;
-        // chord of the support on this row (E <= cut + band) with a margin of 2^-10 + 2^-16 h pixels each
-        // side: the float32 half-chord h is within a few 2^-24 h of its exact value (the guard band of the
-        // exponent already covers the rounding of ey, a0 and the pixel offsets)
-        const float hq_out = sqrt_approx(rem_hi * T.inv_a0);
-        const float h_out = hq_out + fmaf(hq_out, 0x1p-16f, 0x1p-10f);
-        const int c_lo = max(it + (int)ceilf(fx - h_out), i_lo);
-        const int c_hi = min(it + (int)floorf(fx + h_out), i_hi);
-        // interior of the chord (E <= cut - band, same margin): inside for certain, no test
-        int n_lo = c_hi + 1, n_hi = c_hi;
-        const float rem_lo = lim_lo - ey;
-        if (rem_lo > 0.f) {
-          const float hq_in = sqrt_approx(rem_lo * T.inv_a0);
-          const float h_in = hq_in - fmaf(hq_in, 0x1p-16f, 0x1p-10f);
-          if (h_in >= 0.f) {
-            n_lo = max(it + (int)ceilf(fx - h_in), c_lo);
-            n_hi = min(it + (int)floorf(fx + h_in), c_hi);
-            if (n_lo > n_hi) {
-              n_lo = c_hi + 1;
-              n_hi = c_hi;
+        int c_lo, c_hi, n_lo, n_hi;
+        // The chord of the support on this row is [a, b] = fx -+ h, h = sqrt(rem / a0), known to within a margin m:
+        // 2^-13 + 2^-18 h pixels for the float32 arithmetic (its error is below 2^-23 + 2^-21 h) and the guard band of
+        // the exponent, which moves h by at most delta / h where band <= rem / 4.  If no pixel centre lies within m of either end, the
+        // pixels between them are inside for certain and no other is (nearly every row).
+        const float rem = ecut - ey;
+        const float x = rem * inv_a0, q = rsqrtf(x);
+        const float h = x * q;
+        const float m = fmaf(delta, q, fmaf(h, 0x1p-18f, 0x1p-13f));
+        const float a = fx - h, b = fx + h;
+        constexpr float kRint = 12582912.f;  // 1.5 2^23: adding it rounds |v| < 2^22 to the nearest integer
+        const float ta = __fadd_rn(a, kRint), tb = __fadd_rn(b, kRint);
+        const float ra = __fsub_rn(ta, kRint), rb = __fsub_rn(tb, kRint);
+        if (rem >= 4.f * band && fabsf(a - ra) > m && fabsf(b - rb) > m) {
+          const int na = __float_as_int(ta) - 0x4b400000 + (ra < a ? 1 : 0);  // ceil(a)
+          const int nb = __float_as_int(tb) - 0x4b400000 - (rb > b ? 1 : 0);  // floor(b)
+          c_lo = n_lo = max(it + na, i_lo);
+          c_hi = n_hi = min(it + nb, i_hi);
+        } else {
+          // chord of the support with the margin on each side; interior of the chord (E <= cut - band, same
+          // margin): inside for certain, no test; the pixels between are tested one by one
+          const float hq_out = sqrt_approx(rem_hi * inv_a0);
+          const float h_out = hq_out + fmaf(hq_out, 0x1p-16f, 0x1p-10f);
+          c_lo = max(it + (int)ceilf(fx - h_out), i_lo);
+          c_hi = min(it + (int)floorf(fx + h_out), i_hi);
+          n_lo = c_hi + 1;
+          n_hi = c_hi;
+          const float rem_lo = lim_lo - ey;
+          if (rem_lo > 0.f) {
+            const float hq_in = sqrt_approx(rem_lo * inv_a0);
+            const float h_in = hq_in - fmaf(hq_in, 0x1p-16f, 0x1p-10f);
+            if (h_in >= 0.f) {
+              n_lo = max(it + (int)ceilf(fx - h_in), c_lo);
+              n_hi = min(it + (int)floorf(fx + h_in), c_hi);
+              if (n_lo > n_hi) {
+                n_lo = c_hi + 1;
+                n_hi = c_hi;
+              }
             }
           }
         }
@@ -142,10 +204,10 @@ __global__ void __launch_bounds__(kLcThreads) light_curve_kernel(const LcTrack* 
         for (int i = c_lo; i < n_lo; ++i) rim_pixel<PROFILE>(T, k, i, j, it, fx, a0, ey, ecut, band, cut2, row, rw, rm);
         if (PROFILE == 0 && sep) {
           float iw = 0.f, im = 0.f;
-          const float* wx = s_wx + threadIdx.x - i_lo * kLcThreads;
+          const float* wx = s_wx + sid - i_lo * S;
 #pragma unroll 4
           for (int i = n_lo; i <= n_hi; ++i) {
-            const float w = wx[i * kLcThreads];
+            const float w = wx[i * S];
             iw = __fadd_rn(iw, w);
             im = fmaf(w, __ldg(row + i), im);
           }
@@ -164,7 +226,7 @@ __global__ void __launch_bounds__(kLcThreads) light_curve_kernel(const LcTrack* 
             rm = fmaf(w, __ldg(row + i), rm);
             kx = __fadd_rn(kx, 1.f);
           }
-        } else {
+        } else if (n_lo <= n_hi) {
           float acc = 0.f;
 #pragma unroll 4
           for (int i = n_lo; i <= n_hi; ++i) acc = __fadd_rn(acc, __ldg(row + i));
@@ -177,30 +239,67 @@ __global__ void __launch_bounds__(kLcThreads) light_curve_kernel(const LcTrack* 
         acc_two_sum(sm, cm, rm);
       }
     }
-    double m;
+    if (L > 1) {
+      s_part[threadIdx.x] = make_float4(sw, cw, sm, cm);
+      __syncthreads();  // also: every part is done with s_wx and s_sample
+      if (part != 0) continue;
+#pragma unroll
+      for (int p = 1; p < L; ++p) {
+        const float4 o = s_part[threadIdx.x + 32 * p];
+        acc_two_sum(sw, cw, o.x);
+        cw = __fadd_rn(cw, o.y);
+        acc_two_sum(sm, cm, o.z);
+        cm = __fadd_rn(cm, o.w);
+      }
+    }
+    if (g >= n_samples) continue;
+    double mean;
     if (sw > 0.f) {
       // float-float quotient (sm + cm) / (sw + cw): the residual of q sw is exact under fma
       const float q = __fdiv_rn(sm, sw);
       const float r = __fadd_rn(fmaf(-q, sw, sm), fmaf(-q, cw, cm));
-      m = (double)q + (double)__fdiv_rn(r, sw);
+      mean = (double)q + (double)__fdiv_rn(r, sw);
     } else {
-      m = __longlong_as_double(0x7ff8000000000000LL);
+      mean = __longlong_as_double(0x7ff8000000000000LL);
     }
-    mu_out[g] = m;
-    if (dm_out) dm_out[g] = (double)(-2.5f * log10f((float)m));
+    mu_out[g] = mean;
+    if (dm_out) dm_out[g] = (double)(-2.5f * log10f((float)mean));
   }
+}
+
+template <int PROFILE>
+void launch_lc(int parts, const LcTrack* tracks, int n_tracks, int64_t n_samples, double cut2, float ecut,
+               double* mu_out, double* dm_out, int grid, cudaStream_t s) {
+  if (parts == 1)
+    light_curve_kernel<PROFILE, 1><<<grid, kLcThreads, 0, s>>>(tracks, n_tracks, n_samples, cut2, ecut, mu_out, dm_out);
+  else if (parts == 2)
+    light_curve_kernel<PROFILE, 2><<<grid, kLcThreads, 0, s>>>(tracks, n_tracks, n_samples, cut2, ecut, mu_out, dm_out);
+  else if (parts == 4)
+    light_curve_kernel<PROFILE, 4><<<grid, kLcThreads, 0, s>>>(tracks, n_tracks, n_samples, cut2, ecut, mu_out, dm_out);
+  else
+    light_curve_kernel<PROFILE, 8><<<grid, kLcThreads, 0, s>>>(tracks, n_tracks, n_samples, cut2, ecut, mu_out, dm_out);
 }
 
 }  // namespace
 
 namespace rsint {
 
+int lc_parts(int sms, int64_t n_samples, double max_rows) {
+  int parts = 1;
+  while (parts < 8 && n_samples * parts < (int64_t)sms * 4 * kLcThreads && max_rows >= 8.0 * parts) parts *= 2;
+  return parts;
+}
+
 cudaError_t launch_light_curves(int profile, const LcTrack* tracks, int n_tracks, int64_t n_samples, double cut2,
-                                float ecut, double* mu_out, double* dm_out, int grid, cudaStream_t s) {
+                                float ecut, double* mu_out, double* dm_out, int parts, cudaStream_t s) {
+  const int64_t per = kLcThreads / parts;
+  // one CTA per block of samples: supports differ from map to map, and the block scheduler evens them out better
+  // than a fixed stride over a few CTAs per SM does (SMs idle 15 % of the time)
+  const int grid = (int)std::min<int64_t>((n_samples + per - 1) / per, (int64_t)1 << 30);
   if (profile == 0)
-    light_curve_kernel<0><<<grid, kLcThreads, 0, s>>>(tracks, n_tracks, n_samples, cut2, ecut, mu_out, dm_out);
+    launch_lc<0>(parts, tracks, n_tracks, n_samples, cut2, ecut, mu_out, dm_out, grid, s);
   else
-    light_curve_kernel<1><<<grid, kLcThreads, 0, s>>>(tracks, n_tracks, n_samples, cut2, ecut, mu_out, dm_out);
+    launch_lc<1>(parts, tracks, n_tracks, n_samples, cut2, ecut, mu_out, dm_out, grid, s);
   return cudaGetLastError();
 }
 

@@ -253,3 +253,24 @@ def test_large_support_rim_crosses_map(profile, radius):
     tracks = [ri.Track(0, (-100.0 + 0.3, 0.2), (0.0123, 0.0071), 6),
               ri.Track(0, (0.1, 1.0 + 100.0 - 0.4), (0.0031, -0.009), 6)]
     _compare([mu], [w], tracks, profile, radius, f"large support {profile}")
+
+
+@pytest.mark.parametrize("profile,s_pix", [(G, 0.6), (G, 1.2), (G, 2.3), (G, 5.0), (D, 3.2), (D, 6.0), (D, 10.0), (D, 30.0)])
+def test_many_samples_equal_few(profile, s_pix):
+    """A call of many samples runs one thread per sample, calls of few samples share a sample's rows between 1, 2, 4
+    or 8 warps by the support's rows: the same pixels, and means that differ by the rounding of the row sums only
+    ((2 n_r + 10) u each side, as above).  Tracks start and end off the map; one of them has a single sample."""
+    w = _window((150, 131))
+    mp = ri.caustic_map((150, 131), seed=4)
+    pix = (w.hi[0] - w.lo[0]) / 150
+    s = s_pix * pix
+    few = [ri.Track(0, (w.lo[0] - 3 * s, w.lo[1] + 0.4), (0.37 * pix, 0.11 * pix), 421),
+           ri.Track(0, (0.1, w.hi[1] + s), (-0.05 * pix, -0.6 * pix), 257), ri.Track(0, (0.3, 0.2), (0.0, 0.0), 1)]
+    reps = 240                                              # 240 x 679 samples: over 4 x 256 per SM
+    got, _ = _gpu([mp], [w], few, profile, s)
+    many, _ = _gpu([mp], [w], few * reps, profile, s)
+    many = many.reshape(reps, got.size)
+    assert np.array_equal(np.isnan(many), np.broadcast_to(np.isnan(got), many.shape))
+    ok = ~np.isnan(got)
+    n_r = min(2.0 * (6.0 * s if profile == G else s) / pix + 3.0, 150)
+    assert np.abs(many[:, ok] / got[ok] - 1.0).max() <= 2.0 * (2.0 * n_r + 10.0) * U
