@@ -170,10 +170,10 @@ int rs_shoot_rows(rs_field_t f, const rs_ray_grid* g, int64_t row_begin, int64_t
 /*
  * rs_shoot_culled -- rs_shoot_rows that skips rays which provably miss the window: the interactive
  * zoom of Section 4 (a sub-window re-shot at higher resolution only needs the rays that can land
- * in it).  Rays are grouped in cells of 16 x 16; for a cell with ray-box centre c and circumradius
- * rho, the deflection of every ray differs from alpha(c) by at most rho sum_i m_i / (d_i (d_i - rho))
- * (d_i = |c - x_i|), so the cell's source positions lie in a box around lam x - alpha(c); a cell
- * whose box (widened by the float32 error band of its rays and float64 rounding) misses the window
+ * in it).  Rays are grouped in cells of 8 x 8; for a cell with ray-box centre c and circumradius
+ * rho, the deflection of every ray differs from its linear expansion about c by at most rho^2 sum_i m_i /
+ * (d_i^2 (d_i - rho)) (d_i = |c - x_i|), so the cell's source positions lie in a box around lam c - alpha(c); a
+ * cell whose box (widened by the float32 error of its rays and float64 rounding) misses the window
  * is skipped and its rays are counted out of window.  Cells with a lens within 1.02 rho of c are
  * always shot.  Results: the same counts and out-of-window count as rs_shoot_rows, bit for bit (the
  * shot cells use the same per-ray arithmetic and binning, certified binning included).

@@ -757,18 +757,22 @@ int rs_shoot_culled(rs_field_t f, const rs_ray_grid* g, int64_t row_begin, int64
   int64_t n_cx = 0;
   const int64_t n_cells = rsint::cull_cells(d.n_rows, d.n0, &n_cx);
   const int64_t n_coarse = rsint::cull_coarse_cells(d.n_rows, d.n0);
-  // stream-ordered workspace: [re-evaluation count | coarse count | kept count | re-evaluation list |
-  // coarse cell list | cell list]
+  const int64_t n_mid = rsint::cull_mid_cells(d.n_rows, d.n0);
+  // stream-ordered workspace: [re-evaluation count | coarse count | mid count | kept count | re-evaluation list |
+  // coarse cell list | mid cell list | cell list]
   const unsigned cap = g_certify ? rsint::recheck_capacity(d.n_rows * d.n0) : 0u;
   const size_t coarse_off = 32 + sizeof(uint2) * (size_t)cap;
-  const size_t list_off = coarse_off + sizeof(unsigned) * (size_t)n_coarse;
+  const size_t mid_off = coarse_off + sizeof(unsigned) * (size_t)n_coarse;
+  const size_t list_off = mid_off + sizeof(unsigned) * (size_t)n_mid;
   void* ws = nullptr;
   cudaError_t e = dev_alloc_async(&ws, list_off + sizeof(unsigned) * (size_t)n_cells, s);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (culled-shoot workspace)");
   char* base = reinterpret_cast<char*>(ws);
   unsigned* n_coarse_kept = reinterpret_cast<unsigned*>(base + 8);
-  unsigned* n_kept = reinterpret_cast<unsigned*>(base + 16);
+  unsigned* n_mid_kept = reinterpret_cast<unsigned*>(base + 16);
+  unsigned* n_kept = reinterpret_cast<unsigned*>(base + 24);
   unsigned* coarse = reinterpret_cast<unsigned*>(base + coarse_off);
+  unsigned* mid = reinterpret_cast<unsigned*>(base + mid_off);
   unsigned* cells = reinterpret_cast<unsigned*>(base + list_off);
   if (g_certify) {
     d.rc_cap = cap;
@@ -777,10 +781,10 @@ int rs_shoot_culled(rs_field_t f, const rs_ray_grid* g, int64_t row_begin, int64
   }
   e = cudaMemsetAsync(base, 0, 32, s);
   if (e == cudaSuccess)
-    e = rsint::launch_cull(d, w->hi[0], w->hi[1], coarse, n_coarse_kept, cells, n_kept,
+    e = rsint::launch_cull(d, w->hi[0], w->hi[1], coarse, n_coarse_kept, mid, n_mid_kept, cells, n_kept,
                            reinterpret_cast<unsigned long long*>(d_rays_shot), s);
   if (e == cudaSuccess) {
-    const int64_t want = (n_cells + 3) / 4;
+    const int64_t want = (n_cells + 15) / 16;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms(f->device) * 2));
     e = rsint::launch_shoot_cells(d, n_cx, cells, n_kept, grid, s);
   }

@@ -11,18 +11,21 @@
 //   y1 = lam1 c1 - alpha1(c) + (lam1 + q1) h1 + q2 h2 +- rho^2 B,   y2 = lam2 c2 - alpha2(c) + q2 h1 + (lam2 - q1) h2 +- rho^2 B,
 // and sum_i m_i / |x - x_i| <= sum_i m_i / (d_i - rho) = S bounds the rounding of every ray of the cell.  A cell
 // whose box misses the window on some axis is skipped and its rays are counted out of window.  A cell with a lens
-// within 1.02 rho of c has no finite bound and is always shot.  The bound is applied to cells of 64 x 64 rays first
-// and then to the 16 x 16 cells of the kept ones.
+// within 1.02 rho of c has no finite bound and is always shot.  The bound is applied to cells of 64 x 64 rays first,
+// then to the 16 x 16 cells of the kept ones and to the 8 x 8 cells of those.
 //
-// The linear term is what makes the bound worth its cost: without it (|alpha(x) - alpha(c)| <= rho sum m / (d (d -
-// rho))) the x4 zoom of the 1e4-lens map shot 8.52e6 rays for 4.12e6 in the window.
+// x4 zoom of the 1e4-lens map, 4.12e6 rays in the window: 8.52e6 rays shot with cells of 16 x 16 and no linear term
+// (|alpha(x) - alpha(c)| <= rho sum m / (d (d - rho))), 6.78e6 with it -- most of the rest in cells a few rho from a
+// lens, whose area shrinks with the cell's -- hence the cells of 8 x 8.
 #include "rs_internal.h"
 
 namespace {
 
 using namespace rsdev;
 
-constexpr int kCell = 16;        // rays per cell side
+constexpr int kCell = 8;         // rays per side of the cells that are shot
+constexpr int kMid = 16;         // of the second level
+constexpr int kCoarse = 64;      // and of the first
 constexpr int kCullBlock = 256;  // cells per CTA of the bound kernel
 
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -46,12 +49,12 @@ __device__ __forceinline__ void fold(float& hi, float& lo, float p) {
 
 // One thread per cell: the bound sums over all lenses (tiles staged in shared memory), then the
 // cell's source-plane box against the window.  Kept cells are appended to `out`; skipped cells add
-// their rays to the out-of-window count.  Two levels: cells of 64 x 64 rays over the whole call
-// (parent == nullptr), then the 16 cells of 16 x 16 rays of every kept 64 x 64 cell.
-template <int MASS>
+// their rays to the out-of-window count.  The first level takes every cell of the call (parent == nullptr), the
+// others the split x split cells of every kept cell of the level before.
+template <bool MASS>
 __global__ void __launch_bounds__(kCullBlock)
     cull_kernel(const ShootDesc d, int cell_rays, int64_t n_cx, int64_t n_cells, const unsigned* __restrict__ parent,
-                const unsigned* __restrict__ parent_count, int64_t n_px, double hi0, double hi1,
+                const unsigned* __restrict__ parent_count, int64_t n_px, int split, double hi0, double hi1,
                 unsigned* __restrict__ out, unsigned* __restrict__ out_count, unsigned long long* __restrict__ n_shot) {
   __shared__ float4 s_lens[kCullBlock];
   __shared__ float s_mass[kCullBlock];
@@ -60,15 +63,16 @@ __global__ void __launch_bounds__(kCullBlock)
   bool ok;
   if (parent != nullptr) {
     const int64_t pc = *parent_count;
-    if ((int64_t)blockIdx.x * kCullBlock >= pc * 16) return;  // CTA-uniform: no parent cells left
+    const int children = split * split;
+    if ((int64_t)blockIdx.x * kCullBlock >= pc * children) return;  // CTA-uniform: no parent cells left
     const int64_t t = (int64_t)blockIdx.x * kCullBlock + threadIdx.x;
-    const int64_t slot = t >> 4;
-    const int sub = (int)(t & 15);
+    const int64_t slot = t / children;
+    const int sub = (int)(t % children);
     ok = slot < pc;
     const int64_t p = parent[ok ? slot : 0];
     const int64_t py = p / n_px, px = p - py * n_px;
-    cx = px * 4 + (sub & 3);
-    cy = py * 4 + (sub >> 2);
+    cx = px * split + sub % split;
+    cy = py * split + sub / split;
     ok = ok && cx < n_cx && cy < n_cy;
   } else {
     const int64_t c = (int64_t)blockIdx.x * kCullBlock + threadIdx.x;
@@ -129,8 +133,7 @@ __global__ void __launch_bounds__(kCullBlock)
       fold(sh, sl, ps);
     }
   }
-  if (!ok) return;
-  const int64_t rays = (i1 - i0 + 1) * (r1 - r0 + 1);
+  const unsigned rays = ok ? (unsigned)((i1 - i0 + 1) * (r1 - r0 + 1)) : 0u;  // at most 64 x 64
   bool keep = true;
   if (!near) {
     // terms carry a few 2^-22 relative (approximate reciprocal square root and reciprocal, the gap's
@@ -153,39 +156,45 @@ __global__ void __launch_bounds__(kCullBlock)
     const bool finite = isfinite(e1) && isfinite(e2) && isfinite(A1) && isfinite(A2);
     keep = !finite || !(y1 + e1 < d.lo0 || y1 - e1 > hi0 || y2 + e2 < d.lo1 || y2 - e2 > hi1);
   }
-  if (keep) {
-    const unsigned slot = atomicAdd(out_count, 1u);
-    out[slot] = (unsigned)(cy * n_cx + cx);
-    if (n_shot) atomicAdd(n_shot, (unsigned long long)rays);
-  } else if (d.oow) {
-    atomicAdd(d.oow, (unsigned long long)rays);
+  // one append and one count per warp: neighbouring cells stay together in the list
+  const int lane = threadIdx.x & 31;
+  const unsigned kept = __ballot_sync(0xffffffffu, ok && keep);
+  const unsigned shot = __reduce_add_sync(0xffffffffu, keep ? rays : 0u);
+  const unsigned missed = __reduce_add_sync(0xffffffffu, keep ? 0u : rays);
+  unsigned slot = 0;
+  if (lane == 0) {
+    if (kept != 0u) slot = atomicAdd(out_count, (unsigned)__popc(kept));
+    if (n_shot && shot != 0u) atomicAdd(n_shot, (unsigned long long)shot);
+    if (d.oow && missed != 0u) atomicAdd(d.oow, (unsigned long long)missed);
   }
+  slot = __shfl_sync(0xffffffffu, slot, 0);
+  if (ok && keep) out[slot + (unsigned)__popc(kept & ((1u << lane) - 1u))] = (unsigned)(cy * n_cx + cx);
 }
 
-// Kept cells: a CTA of four warps shoots four cells per pass (one per warp); lane l holds row l / 2
-// of its cell and columns 8 (l % 2) .. 8 (l % 2) + 7.  The per-ray arithmetic is rs_shoot's (per-ray
-// squared distances instead of the shared row table give bitwise the same values).
+// Kept cells: a CTA of four warps shoots sixteen cells per pass; eight lanes share a cell, lane l of them holding
+// its row l (eight columns).  The per-ray arithmetic is rs_shoot's (per-ray squared distances instead of the shared
+// row table give bitwise the same values).
 template <int MASS>
 __global__ void __launch_bounds__(128, 2) shoot_cells_kernel(const ShootDesc d, int64_t n_cx,
                                                              const unsigned* __restrict__ list,
                                                              const unsigned* __restrict__ n_kept) {
-  constexpr int RPT = 8;
+  constexpr int RPT = kCell, CELLS = 128 / kCell;
   __shared__ LensSmem<rsint::kTile, 1> sm;
-  __shared__ NearSmem<rsint::kTile, 4, 128, RPT> ns;  // one near-lens box per warp (its cell)
+  __shared__ NearSmem<rsint::kTile, CELLS, 128, RPT> ns;  // one near-lens box per cell
   PipeState ps;
   pipe_init(sm.bar, ps);
   const unsigned count = *n_kept;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (unsigned base = blockIdx.x * 4u; base < count; base += gridDim.x * 4u) {  // CTA-uniform
-    const unsigned slot = base + (unsigned)warp;
+  const int lane = threadIdx.x & 31, own = threadIdx.x / kCell, row = threadIdx.x % kCell;
+  for (unsigned base = blockIdx.x * (unsigned)CELLS; base < count; base += gridDim.x * (unsigned)CELLS) {  // CTA-uniform
+    const unsigned slot = base + (unsigned)own;
     const bool cell_ok = slot < count;
     const int64_t cell = (int64_t)list[cell_ok ? slot : count - 1];
     const int64_t cy = cell / n_cx, cx = cell - cy * n_cx;
-    const int64_t jrel = cy * kCell + (lane >> 1);
+    const int64_t jrel = cy * kCell + row;
     const bool row_ok = cell_ok && jrel < d.n_rows;
     const int64_t j = d.j_begin + (jrel < d.n_rows ? jrel : d.n_rows - 1);
     const float x2r = ray_coord(j, d.sp1, d.or1);
-    const int64_t i_base = cx * kCell + (lane & 1) * RPT;
+    const int64_t i_base = cx * kCell;
     float x1[RPT], x2[RPT];
     bool valid[RPT];
 #pragma unroll
@@ -196,12 +205,26 @@ __global__ void __launch_bounds__(128, 2) shoot_cells_kernel(const ShootDesc d, 
       x1[k] = ray_coord(i, d.sp0, d.or0);
       x2[k] = x2r;
     }
-    if (lane == 0) {
+    if (row == 0) {
       // the cell's ray box (coordinates grow with the grid index)
       const int64_t ia = cx * kCell, ib = min(ia + kCell, d.n0) - 1;
       const int64_t ja = cy * kCell, jb = min(ja + kCell, d.n_rows) - 1;
-      near_set_box(ns, warp, ray_coord(ia, d.sp0, d.or0), ray_coord(ib, d.sp0, d.or0),
+      near_set_box(ns, own, ray_coord(ia, d.sp0, d.or0), ray_coord(ib, d.sp0, d.or0),
                    ray_coord(d.j_begin + ja, d.sp1, d.or1), ray_coord(d.j_begin + jb, d.sp1, d.or1));
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      float u0 = ns.box[0][0], u1 = ns.box[0][1], u2 = ns.box[0][2], u3 = ns.box[0][3];
+      for (int c = 1; c < CELLS; ++c) {
+        u0 = fminf(u0, ns.box[c][0]);
+        u1 = fmaxf(u1, ns.box[c][1]);
+        u2 = fminf(u2, ns.box[c][2]);
+        u3 = fmaxf(u3, ns.box[c][3]);
+      }
+      ns.ubox[0] = u0;
+      ns.ubox[1] = u1;
+      ns.ubox[2] = u2;
+      ns.ubox[3] = u3;
     }
     __syncthreads();  // every box is set before the first lens tile is searched
     float a1h[RPT], a1l[RPT], a2h[RPT], a2l[RPT], sig[RPT], tn[RPT];
@@ -220,31 +243,37 @@ int64_t cull_cells(int64_t n_rows, int64_t n0, int64_t* n_cx) {
   return ((n_rows + kCell - 1) / kCell) * *n_cx;
 }
 
-int64_t cull_coarse_cells(int64_t n_rows, int64_t n0) {
-  constexpr int64_t C = 4 * kCell;
-  return ((n_rows + C - 1) / C) * ((n0 + C - 1) / C);
+static int64_t cells_of(int64_t n_rows, int64_t n0, int side) {
+  return ((n_rows + side - 1) / side) * ((n0 + side - 1) / side);
+}
+int64_t cull_coarse_cells(int64_t n_rows, int64_t n0) { return cells_of(n_rows, n0, kCoarse); }
+int64_t cull_mid_cells(int64_t n_rows, int64_t n0) { return cells_of(n_rows, n0, kMid); }
+
+template <bool MASS>
+static void launch_cull_m(const rsdev::ShootDesc& d, double hi0, double hi1, unsigned* coarse, unsigned* n_coarse,
+                          unsigned* mid, unsigned* n_mid, unsigned* list, unsigned* n_kept, unsigned long long* n_shot,
+                          cudaStream_t s) {
+  const auto across = [&](int side) { return (d.n0 + side - 1) / side; };
+  const auto blocks = [](int64_t cells) { return (unsigned)((cells + kCullBlock - 1) / kCullBlock); };
+  const int64_t n1 = cull_coarse_cells(d.n_rows, d.n0);
+  constexpr int S2 = kCoarse / kMid, S3 = kMid / kCell;
+  // the lower levels are launched for all cells the level above could keep; CTAs beyond what it kept leave at once
+  cull_kernel<MASS><<<blocks(n1), kCullBlock, 0, s>>>(d, kCoarse, across(kCoarse), n1, nullptr, nullptr, 0, 1, hi0, hi1,
+                                                      coarse, n_coarse, nullptr);
+  cull_kernel<MASS><<<blocks(n1 * S2 * S2), kCullBlock, 0, s>>>(d, kMid, across(kMid), 0, coarse, n_coarse,
+                                                                across(kCoarse), S2, hi0, hi1, mid, n_mid, nullptr);
+  cull_kernel<MASS><<<blocks(cull_mid_cells(d.n_rows, d.n0) * S3 * S3), kCullBlock, 0, s>>>(
+      d, kCell, across(kCell), 0, mid, n_mid, across(kMid), S3, hi0, hi1, list, n_kept, n_shot);
 }
 
 cudaError_t launch_cull(const rsdev::ShootDesc& d, double hi0, double hi1, unsigned* coarse, unsigned* n_coarse,
-                        unsigned* list, unsigned* n_kept, unsigned long long* n_shot, cudaStream_t s) {
-  constexpr int64_t C = 4 * kCell;
-  const int64_t n_px = (d.n0 + C - 1) / C;
-  const int64_t n_coarse_cells = cull_coarse_cells(d.n_rows, d.n0);
-  if (n_coarse_cells <= 0) return cudaSuccess;
-  const int64_t n_cx = (d.n0 + kCell - 1) / kCell;
-  const int64_t g1 = (n_coarse_cells + kCullBlock - 1) / kCullBlock;
-  const int64_t g2 = (n_coarse_cells * 16 + kCullBlock - 1) / kCullBlock;
-  if (d.f.has_mass) {
-    cull_kernel<true><<<(unsigned)g1, kCullBlock, 0, s>>>(d, (int)C, n_px, n_coarse_cells, nullptr, nullptr, 0, hi0,
-                                                          hi1, coarse, n_coarse, nullptr);
-    cull_kernel<true><<<(unsigned)g2, kCullBlock, 0, s>>>(d, kCell, n_cx, 0, coarse, n_coarse, n_px, hi0, hi1, list,
-                                                          n_kept, n_shot);
-  } else {
-    cull_kernel<false><<<(unsigned)g1, kCullBlock, 0, s>>>(d, (int)C, n_px, n_coarse_cells, nullptr, nullptr, 0, hi0,
-                                                           hi1, coarse, n_coarse, nullptr);
-    cull_kernel<false><<<(unsigned)g2, kCullBlock, 0, s>>>(d, kCell, n_cx, 0, coarse, n_coarse, n_px, hi0, hi1, list,
-                                                           n_kept, n_shot);
-  }
+                        unsigned* mid, unsigned* n_mid, unsigned* list, unsigned* n_kept, unsigned long long* n_shot,
+                        cudaStream_t s) {
+  if (cull_coarse_cells(d.n_rows, d.n0) <= 0) return cudaSuccess;
+  if (d.f.has_mass)
+    launch_cull_m<true>(d, hi0, hi1, coarse, n_coarse, mid, n_mid, list, n_kept, n_shot, s);
+  else
+    launch_cull_m<false>(d, hi0, hi1, coarse, n_coarse, mid, n_mid, list, n_kept, n_shot, s);
   return cudaGetLastError();
 }
 

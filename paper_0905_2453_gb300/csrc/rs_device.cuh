@@ -275,19 +275,22 @@ struct NoNear {
   static constexpr int kGroups = 1;
 };
 
-// Near-lens search state of a CTA of BLOCK threads holding RPT rays each, whose rays form NG groups
-// (NG = 1: one box around all rays of the CTA; NG = warps: one box per warp).  While a lens tile is
+// Near-lens search state of a CTA of BLOCK threads holding RPT rays each, whose rays form NG groups of
+// consecutive threads (NG = 1: one box around all rays of the CTA; 16: one per 8 threads, a cell).  While a lens tile is
 // being summed, each warp checks its share of the tile's lenses against the boxes and lists the hits
-// (field lens indices) in the list of the tile's parity; the list is evaluated during the next tile,
+// in the list of the tile's parity; the list is evaluated during the next tile,
 // after the end-of-tile barrier that already separates the two, so the search adds no barrier and
 // nothing to the serial part of a tile boundary.
 template <int TILE, int NG, int BLOCK, int RPT>
 struct __align__(16) NearSmem {
   static constexpr bool kOn = true;
   static constexpr int kGroups = NG;
+  static constexpr int kThreads = BLOCK / NG;  // of a group
   float box[NG][4];        // x1 lo, x1 hi, x2 lo, x2 hi of each group's rays, widened by h (rounded outwards)
+  float ubox[4];           // box around all groups' boxes (NG > 1: looked at first)
   int n[2][NG];            // lenses listed per tile parity and group
-  int idx[2][NG][TILE];    // their indices in the field
+  int base[2];             // field index of the first lens of the tile of that parity
+  uint16_t idx[2][NG][TILE];  // the listed lenses' indices in the tile
   float t[RPT * BLOCK];    // per ray: the largest near term so far (thread x's ray k at k * BLOCK + x)
 };
 
@@ -309,11 +312,16 @@ template <int TILE, class NS>
 __device__ __forceinline__ void near_gather(NS& ns, int par, const float4* l4, int cnt, int base, int nwarps) {
   constexpr int NG = NS::kGroups;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) ns.base[par] = base;
   const int share = (TILE + nwarps - 1) / nwarps;
   const int l0 = warp * share, l1 = min(l0 + share, cnt);
   for (int l = l0 + lane; l - lane < l1; l += 32) {  // warp-uniform trip count
     const bool ok = l < l1;
     const float4 L = l4[ok ? l : l0];
+    if constexpr (NG > 1) {
+      const bool any = ok && L.x >= ns.ubox[0] && L.x <= ns.ubox[1] && L.z >= ns.ubox[2] && L.z <= ns.ubox[3];
+      if (__ballot_sync(0xffffffffu, any) == 0u) continue;
+    }
 #pragma unroll
     for (int g = 0; g < NG; ++g) {
       const bool in = ok && L.x >= ns.box[g][0] && L.x <= ns.box[g][1] && L.z >= ns.box[g][2] && L.z <= ns.box[g][3];
@@ -323,7 +331,7 @@ __device__ __forceinline__ void near_gather(NS& ns, int par, const float4* l4, i
         int slot = 0;
         if (lane == leader) slot = atomicAdd(&ns.n[par][g], __popc(mask));
         slot = __shfl_sync(0xffffffffu, slot, leader);
-        if (in) ns.idx[par][g][slot + __popc(mask & ((1u << lane) - 1u))] = base + l;
+        if (in) ns.idx[par][g][slot + __popc(mask & ((1u << lane) - 1u))] = (uint16_t)l;
       }
     }
   }
@@ -345,7 +353,7 @@ __device__ __forceinline__ void near_eval(NS& ns, int par, int g, const FieldDev
 #pragma unroll
   for (int k = 0; k < 2 * NP; ++k) t[k] = ns.t[k * nthreads + threadIdx.x];
   for (int e = 0; e < n; ++e) {
-    const int l = ns.idx[par][g][e];
+    const int l = ns.base[par] + (int)ns.idx[par][g][e];
     const float4 L = __ldg(f.lens4 + l);
     const float m = MASS ? __ldg(f.mass2 + l).x : 1.f;
 #pragma unroll
@@ -734,7 +742,7 @@ __device__ __forceinline__ bool deflect_accumulate(const FieldDev& f, const uint
     }
     if constexpr (NS::kOn) {
       // the previous tile's list is complete (end-of-tile barrier); this tile's share goes to the other list
-      if (t > 0) near_eval<NP, MASS>(*ns, (t - 1) & 1, NS::kGroups == 1 ? 0 : (int)(threadIdx.x >> 5), f, X1, X2,
+      if (t > 0) near_eval<NP, MASS>(*ns, (t - 1) & 1, (int)threadIdx.x / NS::kThreads, f, X1, X2,
                                      (int)blockDim.x);
       near_gather<TILE>(*ns, t & 1, &sm.lens4[b][0], cnt, t * TILE, (int)(blockDim.x >> 5));
     }
@@ -776,7 +784,7 @@ __device__ __forceinline__ bool deflect_accumulate(const FieldDev& f, const uint
   }
   if constexpr (NS::kOn) {
     if (ok && ntiles > 0)  // the last tile's list (complete: end-of-tile barrier)
-      near_eval<NP, MASS>(*ns, (ntiles - 1) & 1, NS::kGroups == 1 ? 0 : (int)(threadIdx.x >> 5), f, X1, X2,
+      near_eval<NP, MASS>(*ns, (ntiles - 1) & 1, (int)threadIdx.x / NS::kThreads, f, X1, X2,
                           (int)blockDim.x);
   }
   if (!ok) {
