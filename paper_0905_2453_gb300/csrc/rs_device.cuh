@@ -38,6 +38,8 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
+
 #include <cuda_runtime.h>
 
 namespace rsdev {
@@ -289,8 +291,9 @@ struct __align__(16) NearSmem {
   float box[NG][4];        // x1 lo, x1 hi, x2 lo, x2 hi of each group's rays, widened by h (rounded outwards)
   float ubox[4];           // box around all groups' boxes (NG > 1: looked at first)
   int n[2][NG];            // lenses listed per tile parity and group
-  int base[2];             // field index of the first lens of the tile of that parity
-  uint16_t idx[2][NG][TILE];  // the listed lenses' indices in the tile
+  int base[2];             // field index of the first lens of the tile of that parity (NG > 1)
+  // the listed lenses' indices in the field (NG = 1) or, to save room, in the tile
+  std::conditional_t<NG == 1, int, uint16_t> idx[2][NG][TILE];
   float t[RPT * BLOCK];    // per ray: the largest near term so far (thread x's ray k at k * BLOCK + x)
 };
 
@@ -312,7 +315,7 @@ template <int TILE, class NS>
 __device__ __forceinline__ void near_gather(NS& ns, int par, const float4* l4, int cnt, int base, int nwarps) {
   constexpr int NG = NS::kGroups;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) ns.base[par] = base;
+  if (NG > 1 && threadIdx.x == 0) ns.base[par] = base;
   const int share = (TILE + nwarps - 1) / nwarps;
   const int l0 = warp * share, l1 = min(l0 + share, cnt);
   for (int l = l0 + lane; l - lane < l1; l += 32) {  // warp-uniform trip count
@@ -331,7 +334,7 @@ __device__ __forceinline__ void near_gather(NS& ns, int par, const float4* l4, i
         int slot = 0;
         if (lane == leader) slot = atomicAdd(&ns.n[par][g], __popc(mask));
         slot = __shfl_sync(0xffffffffu, slot, leader);
-        if (in) ns.idx[par][g][slot + __popc(mask & ((1u << lane) - 1u))] = (uint16_t)l;
+        if (in) ns.idx[par][g][slot + __popc(mask & ((1u << lane) - 1u))] = NG == 1 ? base + l : l;
       }
     }
   }
@@ -353,7 +356,7 @@ __device__ __forceinline__ void near_eval(NS& ns, int par, int g, const FieldDev
 #pragma unroll
   for (int k = 0; k < 2 * NP; ++k) t[k] = ns.t[k * nthreads + threadIdx.x];
   for (int e = 0; e < n; ++e) {
-    const int l = ns.base[par] + (int)ns.idx[par][g][e];
+    const int l = (NS::kGroups > 1 ? ns.base[par] : 0) + (int)ns.idx[par][g][e];
     const float4 L = __ldg(f.lens4 + l);
     const float m = MASS ? __ldg(f.mass2 + l).x : 1.f;
 #pragma unroll
