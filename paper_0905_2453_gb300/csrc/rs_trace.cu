@@ -171,14 +171,15 @@ __global__ void __launch_bounds__(128)
 
 // Folds the ng groups of a chunk (first: group g0 of the field) into the accumulators of ray pair (block, q) =
 // blockIdx.x: warp 0 the first axis, warp 1 the second, warp 2 the band sums.  Serial in the groups, so bound by
-// latency: sixteen groups are loaded while the sixteen before them are folded.  The last chunk ends in the
-// outputs.
+// latency: a ring in shared memory keeps 64 groups in flight ahead of the fold.  The last chunk ends in the outputs.
 __global__ void __launch_bounds__(96)
     trace_fold_kernel(const FieldDev f, int64_t n_rb, int g0, int ng, const uint64_t* __restrict__ part,
                       uint64_t* __restrict__ state, int last, const float2* __restrict__ xy,
                       const float* __restrict__ tmax, int64_t k, double* __restrict__ y, double* __restrict__ alpha,
                       double* __restrict__ err) {
-  constexpr int AHEAD = 16;  // a multiple of the renormalisation period (four groups)
+  constexpr int AHEAD = 16;   // groups of a stage: a multiple of the renormalisation period (four groups)
+  constexpr int STAGES = 5;   // stages of the ring, all but one in flight
+  __shared__ __align__(16) uint64_t ring[STAGES][AHEAD][64];  // [group][P1 of 32 lanes, P2 of 32 lanes]
   __shared__ uint64_t s_acc[kStateWords][32];
   const int role = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t rb = (int64_t)blockIdx.x >> 1;
@@ -189,38 +190,50 @@ __global__ void __launch_bounds__(96)
     a = st[0];
     b = st[32];
   }
-  const uint64_t* p = part + (size_t)rb * 128 + q * 64 + lane;
+  const uint64_t* p = part + (size_t)rb * 128 + q * 64;
   const size_t step = (size_t)n_rb * 128;
   const int whole = min(ng, f.n_lens / kGroup - g0);  // whole groups of the chunk: renormalised as in the shoot
-  uint64_t u[AHEAD], v[AHEAD];
-  auto load = [&](int g) {
-#pragma unroll
-    for (int j = 0; j < AHEAD; ++j) {
-      const uint64_t* pj = p + (size_t)min(g + j, ng - 1) * step;
-      u[j] = __ldcg(reinterpret_cast<const unsigned long long*>(pj + (role == 1 ? 32 : 0)));
-      v[j] = role == 2 ? __ldcg(reinterpret_cast<const unsigned long long*>(pj + 32)) : 0ull;
+  auto fetch = [&](int stage) {
+    for (int i = threadIdx.x; i < AHEAD * 32; i += 96) {  // 16-byte pieces, 32 a group
+      const int g = stage * AHEAD + i / 32;
+      if (g < ng)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         smem_u32(&ring[stage % STAGES][i / 32][2 * (i % 32)])),
+                     "l"(p + (size_t)g * step + 2 * (i % 32))
+                     : "memory");
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  load(0);
-  for (int g = 0; g < ng; g += AHEAD) {
-    uint64_t cu[AHEAD], cv[AHEAD];
+  for (int t = 0; t < STAGES - 1; ++t) fetch(t);
+  for (int t = 0; t * AHEAD < ng; ++t) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+    __syncthreads();        // stage t has arrived, and every warp is done with stage t - 1
+    fetch(t + STAGES - 1);  // into the slot of stage t - 1
+    const uint64_t(*u)[64] = ring[t % STAGES];
+    const int g = t * AHEAD;
+    auto band = [&](int j) {
+      const uint64_t p1 = u[j][lane], p2 = u[j][32 + lane];
+      a = f2_fma(p1, p1, a);
+      a = f2_fma(p2, p2, a);
+      b = f2_add_x(b, f2_add_x(f2_abs(p1), f2_abs(p2)));
+    };
+    auto axis = [&](int j, bool renorm) {
+      twosum_accumulate(a, b, u[j][role * 32 + lane]);
+      if (renorm) renormalise(a, b);
+    };
+    // a whole stage has no branch between its groups, so that their additions overlap
+    if (g + AHEAD > whole) {
+      for (int j = 0; j < AHEAD && g + j < ng; ++j)
+        if (role == 2)
+          band(j);
+        else
+          axis(j, (j & 3) == 3 && g + j < whole);
+    } else if (role == 2) {
 #pragma unroll
-    for (int j = 0; j < AHEAD; ++j) {
-      cu[j] = u[j];
-      cv[j] = v[j];
-    }
-    if (g + AHEAD < ng) load(g + AHEAD);  // in flight while this block is folded
+      for (int j = 0; j < AHEAD; ++j) band(j);
+    } else {
 #pragma unroll
-    for (int j = 0; j < AHEAD; ++j) {
-      if (g + j >= ng) break;
-      if (role == 2) {
-        a = f2_fma(cu[j], cu[j], a);
-        a = f2_fma(cv[j], cv[j], a);
-        b = f2_add_x(b, f2_add_x(f2_abs(cu[j]), f2_abs(cv[j])));
-      } else {
-        twosum_accumulate(a, b, cu[j]);
-        if ((j & 3) == 3 && g + j < whole) renormalise(a, b);
-      }
+      for (int j = 0; j < AHEAD; ++j) axis(j, (j & 3) == 3);
     }
   }
   if (!last) {
