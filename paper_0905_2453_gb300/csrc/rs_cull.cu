@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kCullBlock)
   const double h1 = fmax((double)c1 - (double)xa1, (double)xb1 - (double)c1);
   const double h2 = fmax((double)c2 - (double)xa2, (double)xb2 - (double)c2);
   const float rho = (float)(sqrt(h1 * h1 + h2 * h2) * (1.0 + 0x1p-20)) + 1e-30f;
-  const float rho_near = 1.02f * rho;  // d <= 1.02 rho: no usable bound
+  const float rho_gap = 0.02f * rho;  // d - rho <= 0.02 rho: no usable bound
   float a1h = 0.f, a1l = 0.f, a2h = 0.f, a2l = 0.f, bh = 0.f, bl = 0.f, sh = 0.f, sl = 0.f;
   float q1h = 0.f, q1l = 0.f, q2h = 0.f, q2l = 0.f;
   bool near = false;
@@ -99,31 +99,40 @@ __global__ void __launch_bounds__(kCullBlock)
     const int l = t0 + threadIdx.x;
     if (l < n) {
       s_lens[threadIdx.x] = d.f.lens4[l];
-      s_mass[threadIdx.x] = MASS ? d.f.mass2[l].x : 1.f;
+      if (MASS) s_mass[threadIdx.x] = d.f.mass2[l].x;
     }
     __syncthreads();
     const int cnt = min(kCullBlock, n - t0);
     for (int g = 0; g < cnt; g += 32) {
       float pa1 = 0.f, pa2 = 0.f, pb = 0.f, ps = 0.f, pq1 = 0.f, pq2 = 0.f;
-      const int ge = min(g + 32, cnt);
-      for (int q = g; q < ge; ++q) {
+      auto term = [&](int q) {
         const float4 L = s_lens[q];
-        const float m = s_mass[q];
         const float dx = c1 - L.x, dy = c2 - L.z;
-        const float d2 = fmaf(dx, dx, dy * dy);
+        const float dy2 = dy * dy;
+        const float d2 = fmaf(dx, dx, dy2);
         const float rs = rsqrt_approx(d2);
-        const float dist = d2 * rs;
-        near |= !(dist > rho_near);  // NaN (a lens on the centre) counts as near
+        const float gap = fmaf(d2, rs, -rho);  // d - rho
+        near |= !(gap > rho_gap);  // NaN (a lens on the centre) counts as near
         const float r2 = rs * rs;
-        const float mi = m * r2;
+        float mi = r2, mg = rcp_approx(gap);
+        if (MASS) {
+          const float m = s_mass[q];
+          mi *= m;
+          mg *= m;
+        }
         pa1 = fmaf(mi, dx, pa1);
         pa2 = fmaf(mi, dy, pa2);
         const float mq = mi * r2;
-        pq1 = fmaf(mq, fmaf(dx, dx, -(dy * dy)), pq1);
+        pq1 = fmaf(mq, fmaf(dx, dx, -dy2), pq1);
         pq2 = fmaf(mq, dx * dy, pq2);
-        const float mg = m * rcp_approx(dist - rho);
         ps += mg;
         pb = fmaf(mg, r2, pb);
+      };
+      if (g + 32 <= cnt) {
+#pragma unroll 8
+        for (int q = g; q < g + 32; ++q) term(q);
+      } else {
+        for (int q = g; q < cnt; ++q) term(q);
       }
       fold(a1h, a1l, pa1);
       fold(a2h, a2l, pa2);
