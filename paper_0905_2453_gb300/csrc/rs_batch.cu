@@ -10,18 +10,10 @@ namespace {
 
 using namespace rsdev;
 
-// MINB resident CTAs per SM as the occupancy floor, as for the plain kernel, except three: the
-// launch shapes compiled for three CTAs per SM (168 registers) run here as their two-CTA twins.
-// Inside the item loop the 168-register build of the tile body ran 1.6-3 % slower than the plain
-// kernel's (one-field batches of 1e3-1e5 lenses), whatever held the descriptor (shared memory,
-// kernel parameter, constant bank, global) and with the tile body out of line; at two CTAs per SM
-// (up to 255 registers) the batch kernel matches the plain one.  The four-CTA shape (4 rays per
-// thread, 128 registers) is for small fields, whose batches it speeds up by a third.  Counts do not
-// depend on the shape.
-template <int MINB>
-constexpr int batch_minb() {
-  return MINB == 3 ? 2 : MINB;
-}
+// MINB resident CTAs per SM as the occupancy floor, as for the plain kernel.  (With one grid row per thread the
+// 168-register build of the three-CTA shapes ran 1.6-3 % behind the plain kernel here and gave way to the two-CTA
+// build; with two rows it is the faster one, 16 uneven fields of 100 to 30000 lenses 40.68 -> 40.29 ms.)  Counts do
+// not depend on the shape.
 template <int WARPS, int RPT, int TILE, int MASS, int MINB>
 __global__ void __launch_bounds__(WARPS * 32, MINB)
     batch_kernel(const ShootDesc* __restrict__ descs, const int2* __restrict__ items, int n_items, int* counter) {
@@ -96,7 +88,7 @@ cudaError_t launch_batch(int cfg, int mass, const rsdev::ShootDesc* descs, const
   switch (cfg) {
 #define RS_CASE(i, w, r, t, m) \
   case i:                       \
-    return launch_batch_t<w, r, t, batch_minb<m>()>(mass, descs, items, n_items, counter, grid, s);
+    return launch_batch_t<w, r, t, m>(mass, descs, items, n_items, counter, grid, s);
     RS_LAUNCH_SHAPES(RS_CASE)
 #undef RS_CASE
     default: return cudaErrorInvalidValue;
@@ -108,7 +100,7 @@ cudaError_t batch_blocks_per_sm(int cfg, int mass, int* blocks) {
   switch (cfg) {
 #define RS_CASE(i, w, r, t, m) \
   case i:                       \
-    return occ_t<w, r, t, batch_minb<m>()>(mass, blocks);
+    return occ_t<w, r, t, m>(mass, blocks);
     RS_LAUNCH_SHAPES(RS_CASE)
 #undef RS_CASE
     default: return cudaErrorInvalidValue;
