@@ -35,6 +35,8 @@
  *     the pairs (three of every four with unit masses, every other pair with
  *     per-lens masses) one reciprocal of the product of the two squared
  *     distances serves both lenses (Montgomery's simultaneous inversion).
+ *     Masses multiply the distances, (m d) / r^2 (fields with a mass above 2^64:
+ *     (m / r^2) d).
  *     Per ray, partial sums over consecutive groups of 64 lenses (in lens index
  *     order) are folded into a two-float (hi, lo) accumulator with an
  *     error-free TwoSum; (hi, lo) is renormalised after every 256 lenses.  With
@@ -259,7 +261,10 @@ int rs_partition_recheck(rs_field_t part, int weighted, const rs_ray_grid* g, in
  *   d_err    : double[2*k] device or NULL, receives per axis the half-width of the band
  *              around y inside which the float32 result cannot decide a pixel (see
  *              certified binning below); asking for it costs one more pass over the lenses.
- * The per-ray arithmetic is the one rs_shoot uses, bit for bit (the band included).
+ * The per-ray arithmetic is the one rs_shoot uses, bit for bit (the band included).  Few rays
+ * through many lenses take a stream-ordered workspace (at most 32 MiB + 36 bytes per ray) to sum a
+ * ray's lens groups side by side; where it cannot be had, and while the stream is being captured,
+ * the call runs without it, slower and with the same bits.
  */
 int rs_trace(rs_field_t f, const rs_ray_grid* g, const int64_t* d_ray_ij, int64_t k, double* d_y,
              double* d_alpha, double* d_err, void* stream);

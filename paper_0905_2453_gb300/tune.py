@@ -196,7 +196,7 @@ def batch_shapes(fields, grids, windows, stream=None, cache_path: str = None, **
     """A launch shape per field of a batch: fields are grouped by mass mode and lens-count bucket (the cache
     key's), the largest field (most rays) of each group is tuned, and its shape serves the group.  Returns a list
     of (block, rpt, lens_tile, min_ctas) for rs_batch_create_shaped.  The launch configuration of each mass mode is left as
-    it was."""
+    rs_get_launch_config reported it (set, where the library chose shapes by size before)."""
     from . import rs_get_launch_config
     saved = {m: rs_get_launch_config(m) for m in (False, True)}
     groups = {}
