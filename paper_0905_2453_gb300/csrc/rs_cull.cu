@@ -1,5 +1,5 @@
 // Culled shooting (the interactive zoom of Section 4: a sub-window of the source plane re-shot at
-// higher resolution): rays are grouped in cells of 16 x 16; a cell is skipped when a rigorous bound
+// higher resolution): rays are grouped in cells of 8 x 8; a cell is skipped when a rigorous bound
 // shows that none of its rays can land in the window, and the others are shot with the same per-ray
 // arithmetic as rs_shoot, so the counts and the out-of-window count equal those of rs_shoot.
 //
