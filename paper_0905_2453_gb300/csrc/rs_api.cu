@@ -355,7 +355,7 @@ extern "C" {
 
 const char* rs_last_error(void) { return g_err.c_str(); }
 
-const char* rs_version(void) { return "rs-gb300 0.4 (sm_103a)"; }
+const char* rs_version(void) { return "rs-gb300 0.5 (sm_103a)"; }
 
 int rs_device_code_version(int* binary_version) {
   if (!binary_version) return fail(RS_EINVAL, "binary_version is NULL");
