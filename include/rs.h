@@ -360,9 +360,11 @@ int rs_field_status(rs_field_t f, int clear, int* status);
  * rs_set_launch_config selects the shape used by rs_shoot / rs_shoot_rows /
  * rs_shoot_rows_noalloc (and by batches planned afterwards) for fields without
  * (has_masses = 0) or with per-lens masses; RS_EINVAL for a shape that is not
- * compiled.  Until it is called for a mass mode the library takes a shape per call by the
- * number of lenses and rays (batches: by the number of lenses of each field), and
- * rs_get_launch_config reports 128 x 8 x 512 at two CTAs per SM.  rs_launch_configs lists the compiled shapes: up to `cap`
+ * compiled.  Until it is called for a mass mode, and again after rs_unset_launch_config, the
+ * library takes a shape per call by the number of lenses and rays (batches: by the number of
+ * lenses of each field); rs_get_launch_config then reports 128 x 8 x 512 at two CTAs per SM and
+ * rs_launch_config_is_set reports 0 (1 once a shape was set): a caller that sets a shape for a
+ * while puts back what was there with either of the two.  rs_launch_configs lists the compiled shapes: up to `cap`
  * (block, rpt, lens_tile, min_ctas) quadruples into `shapes` (int[4*cap]);
  * returns the number available via *count.  rs_launch_occupancy reports how
  * many CTAs of a shape's shoot kernel are resident per SM on the current device
@@ -370,6 +372,8 @@ int rs_field_status(rs_field_t f, int clear, int* status);
  */
 int rs_set_launch_config(int has_masses, int block, int rays_per_thread, int lens_tile, int min_ctas);
 int rs_get_launch_config(int has_masses, int* block, int* rays_per_thread, int* lens_tile, int* min_ctas);
+int rs_unset_launch_config(int has_masses);
+int rs_launch_config_is_set(int has_masses, int* is_set);
 int rs_launch_configs(int* shapes, int cap, int* count);
 int rs_launch_occupancy(int has_masses, int block, int rays_per_thread, int lens_tile, int min_ctas,
                         int* ctas_per_sm);

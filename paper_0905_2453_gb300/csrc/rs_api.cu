@@ -385,6 +385,18 @@ int rs_get_launch_config(int has_masses, int* block, int* rays_per_thread, int* 
   return RS_OK;
 }
 
+int rs_unset_launch_config(int has_masses) {
+  g_cfg[has_masses ? 1 : 0] = rsint::kDefaultCfg;
+  g_cfg_set[has_masses ? 1 : 0] = false;
+  return RS_OK;
+}
+
+int rs_launch_config_is_set(int has_masses, int* is_set) {
+  if (!is_set) return fail(RS_EINVAL, "is_set is NULL");
+  *is_set = g_cfg_set[has_masses ? 1 : 0] ? 1 : 0;
+  return RS_OK;
+}
+
 int rs_launch_occupancy(int has_masses, int block, int rays_per_thread, int lens_tile, int min_ctas,
                         int* ctas_per_sm) {
   if (!ctas_per_sm) return fail(RS_EINVAL, "ctas_per_sm is NULL");

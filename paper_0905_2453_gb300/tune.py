@@ -16,13 +16,15 @@ would take minutes per shape.
 """
 from __future__ import annotations
 
+import contextlib
 import json
 import math
 import os
 
 import torch
 
-from . import rs_launch_configs, rs_launch_occupancy, rs_set_launch_config, rs_shoot_rows, rs_version
+from . import (rs_get_launch_config, rs_launch_config_is_set, rs_launch_configs, rs_launch_occupancy,
+               rs_set_launch_config, rs_shoot_rows, rs_unset_launch_config, rs_version)
 
 DEFAULT_CACHE = os.path.join(os.environ.get("XDG_CACHE_HOME", os.path.expanduser("~/.cache")),
                              "rs_gb300", "tune.json")
@@ -192,25 +194,34 @@ def autotune(field, grid, window, min_rays: float = 8e6, max_interactions: float
     return (*sh, timings)
 
 
+@contextlib.contextmanager
+def kept_launch_configs():
+    """Puts the launch configuration of both mass modes back at the end: the shape that was set, or shapes by size."""
+    saved = {m: rs_get_launch_config(m) if rs_launch_config_is_set(m) else None for m in (False, True)}
+    try:
+        yield
+    finally:
+        for m, sh in saved.items():
+            if sh is None:
+                rs_unset_launch_config(m)
+            else:
+                rs_set_launch_config(m, *sh)
+
+
 def batch_shapes(fields, grids, windows, stream=None, cache_path: str = None, **kw):
     """A launch shape per field of a batch: fields are grouped by mass mode and lens-count bucket (the cache
     key's), the largest field (most rays) of each group is tuned, and its shape serves the group.  Returns a list
-    of (block, rpt, lens_tile, min_ctas) for rs_batch_create_shaped.  The launch configuration of each mass mode is left as
-    rs_get_launch_config reported it (set, where the library chose shapes by size before)."""
-    from . import rs_get_launch_config
-    saved = {m: rs_get_launch_config(m) for m in (False, True)}
+    of (block, rpt, lens_tile, min_ctas) for rs_batch_create_shaped.  The launch configuration of each mass mode is
+    left as it was."""
     groups = {}
     for k, (f, g) in enumerate(zip(fields, grids)):
         n_lens, has_mass = f.info()
         groups.setdefault((int(has_mass), _bucket(n_lens)), []).append(k)
     shapes = [None] * len(fields)
-    try:
+    with kept_launch_configs():
         for members in groups.values():
             big = max(members, key=lambda k: int(grids[k].n[0]) * int(grids[k].n[1]))
             sh = tuple(autotune(fields[big], grids[big], windows[big], stream=stream, cache_path=cache_path, **kw)[:4])
             for k in members:
                 shapes[k] = sh
-    finally:
-        for m, sh in saved.items():
-            rs_set_launch_config(m, *sh)
     return shapes

@@ -28,3 +28,13 @@ def pytest_collection_modifyitems(config, items):
     for it in items:
         if "gpu" in it.keywords:
             it.add_marker(skip)
+
+
+@pytest.fixture(autouse=True)
+def _shapes_by_size():
+    """Every test starts with launch shapes taken by size, whatever shape the test before it set."""
+    yield
+    rs = sys.modules.get("paper_0905_2453_gb300")
+    if rs is not None and getattr(rs, "_lib", None) is not None:
+        for m in (False, True):
+            rs.rs_unset_launch_config(m)

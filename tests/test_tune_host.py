@@ -73,3 +73,21 @@ def test_batch_shapes_tune_the_largest_field_of_each_mass_mode_and_lens_bucket(m
     assert sorted(tuned) == sorted([(110, False, 2048), (100, True, 1024), (11000, True, 4096)])
     assert shapes == [(128, 4, 256, 4)] * 3 + [(128, 8, 512, 3)] * 2 + [(128, 4, 256, 4)]
     assert {m: rs.rs_get_launch_config(m) for m in (False, True)} == before
+    assert not rs.rs_launch_config_is_set(False) and not rs.rs_launch_config_is_set(True)  # shapes by size still
+
+
+def test_launch_configs_are_put_back_set_or_by_size():
+    import paper_0905_2453_gb300 as rs
+    from paper_0905_2453_gb300 import tune
+    default = rs.rs_get_launch_config(False)
+    rs.rs_set_launch_config(True, 128, 8, 256, 3)
+    assert not rs.rs_launch_config_is_set(False) and rs.rs_launch_config_is_set(True)
+    with pytest.raises(ZeroDivisionError), tune.kept_launch_configs():
+        rs.rs_set_launch_config(False, 128, 4, 256, 4)
+        rs.rs_unset_launch_config(True)
+        assert rs.rs_launch_config_is_set(False) and not rs.rs_launch_config_is_set(True)
+        1 / 0
+    assert not rs.rs_launch_config_is_set(False) and rs.rs_get_launch_config(False) == default
+    assert rs.rs_launch_config_is_set(True) and rs.rs_get_launch_config(True) == (128, 8, 256, 3)
+    rs.rs_unset_launch_config(True)
+    assert not rs.rs_launch_config_is_set(True) and rs.rs_get_launch_config(True) == default
