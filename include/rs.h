@@ -364,7 +364,8 @@ int rs_field_status(rs_field_t f, int clear, int* status);
  * library takes a shape per call by the number of lenses and rays (batches: by the number of
  * lenses of each field); rs_get_launch_config then reports 128 x 8 x 512 at two CTAs per SM and
  * rs_launch_config_is_set reports 0 (1 once a shape was set): a caller that sets a shape for a
- * while puts back what was there with either of the two.  rs_launch_configs lists the compiled shapes: up to `cap`
+ * while puts back what was there with either of the two.  rs_launch_config_by_size reports the shape
+ * so taken for n_rows x n0 rays through n_lens lenses on a device of sms SMs.  rs_launch_configs lists the compiled shapes: up to `cap`
  * (block, rpt, lens_tile, min_ctas) quadruples into `shapes` (int[4*cap]);
  * returns the number available via *count.  rs_launch_occupancy reports how
  * many CTAs of a shape's shoot kernel are resident per SM on the current device
@@ -374,6 +375,8 @@ int rs_set_launch_config(int has_masses, int block, int rays_per_thread, int len
 int rs_get_launch_config(int has_masses, int* block, int* rays_per_thread, int* lens_tile, int* min_ctas);
 int rs_unset_launch_config(int has_masses);
 int rs_launch_config_is_set(int has_masses, int* is_set);
+int rs_launch_config_by_size(int has_masses, int64_t n_lens, int64_t n_rows, int64_t n0, int sms, int* block,
+                             int* rays_per_thread, int* lens_tile, int* min_ctas);
 int rs_launch_configs(int* shapes, int cap, int* count);
 int rs_launch_occupancy(int has_masses, int block, int rays_per_thread, int lens_tile, int min_ctas,
                         int* ctas_per_sm);

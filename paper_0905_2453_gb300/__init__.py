@@ -29,7 +29,7 @@ __all__ = [
     "rs_create_field", "rs_destroy_field", "rs_field_info", "rs_shoot", "rs_shoot_rows", "rs_trace",
     "rs_magnification", "rs_batch_create", "rs_batch_launch", "rs_batch_destroy", "rs_shoot_batch",
     "rs_field_status", "rs_last_error", "rs_version", "rs_set_launch_config", "rs_get_launch_config",
-    "rs_unset_launch_config", "rs_launch_config_is_set", "rs_launch_configs", "rs_trace_certified", "rs_set_certified_binning", "rs_get_certified_binning",
+    "rs_unset_launch_config", "rs_launch_config_is_set", "rs_launch_config_by_size", "rs_launch_configs", "rs_trace_certified", "rs_set_certified_binning", "rs_get_certified_binning",
     "rs_selftest_bounded_wait", "rs_shoot_rows_noalloc", "rs_light_curves", "rs_shoot_culled",
     "rs_create_moving_field", "rs_field_set_time", "rs_field_time", "rs_shoot_staged", "rs_shoot_streamed",
     "rs_set_staged_state_budget", "rs_set_alloc_failure", "rs_light_curve_plan_create", "rs_light_curve_plan_samples",
@@ -44,7 +44,7 @@ EXPORTED_SYMBOLS = (
     "rs_create_field", "rs_destroy_field", "rs_field_info", "rs_shoot", "rs_shoot_rows", "rs_trace",
     "rs_magnification", "rs_batch_create", "rs_batch_launch", "rs_batch_destroy", "rs_shoot_batch",
     "rs_field_status", "rs_last_error", "rs_version", "rs_set_launch_config", "rs_get_launch_config",
-    "rs_unset_launch_config", "rs_launch_config_is_set", "rs_launch_configs", "rs_trace_certified", "rs_set_certified_binning", "rs_get_certified_binning",
+    "rs_unset_launch_config", "rs_launch_config_is_set", "rs_launch_config_by_size", "rs_launch_configs", "rs_trace_certified", "rs_set_certified_binning", "rs_get_certified_binning",
     "rs_selftest_bounded_wait", "rs_shoot_rows_noalloc", "rs_light_curves", "rs_shoot_culled",
     "rs_create_moving_field", "rs_field_set_time", "rs_field_time", "rs_shoot_staged", "rs_shoot_streamed",
     "rs_set_staged_state_budget", "rs_set_alloc_failure",
@@ -164,6 +164,7 @@ def load():
         "rs_get_launch_config": ([i32] + [ctypes.POINTER(i32)] * 4, i32),
         "rs_unset_launch_config": ([i32], i32),
         "rs_launch_config_is_set": ([i32, ctypes.POINTER(i32)], i32),
+        "rs_launch_config_by_size": ([i32, i64, i64, i64, i32] + [ctypes.POINTER(i32)] * 4, i32),
         "rs_launch_configs": ([ctypes.POINTER(i32), i32, ctypes.POINTER(i32)], i32),
         "rs_launch_occupancy": ([i32, i32, i32, i32, i32, ctypes.POINTER(i32)], i32),
         "rs_partition_buffer_bytes": ([gp, i64, i64, ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(ctypes.c_uint64),
@@ -679,6 +680,15 @@ def rs_launch_config_is_set(has_masses: bool) -> bool:
     v = ctypes.c_int(0)
     _check(load().rs_launch_config_is_set(1 if has_masses else 0, ctypes.byref(v)), "rs_launch_config_is_set")
     return bool(v.value)
+
+
+def rs_launch_config_by_size(has_masses: bool, n_lens: int, n_rows: int, n0: int, sms: int):
+    """(block, rays_per_thread, lens_tile, min_ctas) of a call of n_rows x n0 rays through n_lens lenses on sms SMs
+    while no shape is set."""
+    v = [ctypes.c_int() for _ in range(4)]
+    _check(load().rs_launch_config_by_size(1 if has_masses else 0, int(n_lens), int(n_rows), int(n0), int(sms),
+                                           *[ctypes.byref(x) for x in v]), "rs_launch_config_by_size")
+    return tuple(int(x.value) for x in v)
 
 
 def rs_launch_configs():

@@ -105,6 +105,55 @@ __global__ void selftest_wait_kernel(uint64_t limit_ns, unsigned int* out) {
 
 }  // namespace
 
+namespace rsint {
+
+// What an SM needs for its share of a call's CTAs.  A call ends with the SM that got most of them, s = ceil(CTAs /
+// SMs), and until more are resident than a shape is compiled for, s is also how many of them hide one another's
+// latency.  ns per lens for s = 1 .. 4 and for each one after (grids of exactly s CTAs per SM through 1e5 lenses),
+// unit masses and per-lens masses; ns per CTA for its start and its rays' epilogue (100 to 1000 lenses).
+//
+// The choice against 128x8x512 at two CTAs per SM on 520 squares and row blocks of 4 to 256 rows, 60 to 60000 lenses:
+// 1.4 % behind at most (800 columns, the last tile all but empty), 5 % to a third ahead below 768 lenses and where
+// large CTAs leave an SM's share uneven, us (two-CTA / chosen): 1e4 lenses x 288^2 394 / 376, x 640^2 1161 / 941,
+// x 8192 x 64 1164 / 1076, 6e4 x 512^2 3646 / 3646, 120 x 1000^2 64 / 54.  Three CTAs per SM whatever the share, as
+// below one large CTA per SM, is up to 7.5 % behind (2048 x 40 rays, 6e4 lenses).
+struct ShapeCost {
+  int cfg;
+  double lens[2][5];
+  double cta;
+};
+constexpr ShapeCost kShapeCosts[] = {
+    {8, {{31.9, 57.4, 84.7, 111.3, 26.9}, {35.7, 60.6, 91.4, 118.6, 28.7}}, 4500.0},   // 128x8x512, two CTAs per SM
+    {10, {{34.5, 57.8, 84.2, 110.9, 26.4}, {37.4, 62.5, 90.3, 119.5, 28.2}}, 3400.0},  // 128x8x512, three
+    {7, {{19.0, 31.8, 47.3, 61.5, 14.7}, {21.4, 33.7, 52.6, 66.7, 16.1}}, 1500.0},     // 128x4x512, two
+    {11, {{21.4, 32.4, 46.7, 60.6, 14.1}, {23.1, 34.0, 49.0, 63.9, 15.0}}, 1150.0},    // 128x4x256, four
+};
+static_assert(kCfgs[8].rpt == 8 && kCfgs[8].tile == 512 && kCfgs[8].min_ctas == 2 && kCfgs[10].rpt == 8 &&
+                  kCfgs[10].tile == 512 && kCfgs[10].min_ctas == 3 && kCfgs[7].rpt == 4 && kCfgs[7].tile == 512 &&
+                  kCfgs[7].min_ctas == 2 && kCfgs[11].rpt == 4 && kCfgs[11].tile == 256 && kCfgs[11].min_ctas == 4,
+              "the shapes that kShapeCosts was measured with");
+
+int shape_by_size(bool masses, double n_lens, int64_t n_rows, int64_t n0, int sms) {
+  int best = kDefaultCfg;
+  double least = INFINITY;
+  for (const ShapeCost& c : kShapeCosts) {
+    const KernelCfg& k = kCfgs[c.cfg];
+    const int64_t warps = k.block / 32, seg = 32 * (int64_t)k.rpt;
+    const double ctas = (double)((n_rows + warps - 1) / warps) * (double)((n0 + seg - 1) / seg);
+    const double share = std::max(1.0, std::ceil(ctas / std::max(1, sms)));
+    const double* t = c.lens[masses ? 1 : 0];
+    const double per_lens = share <= 4.0 ? t[(int)share - 1] : t[3] + (share - 4.0) * t[4];
+    const double cost = per_lens * n_lens + c.cta * share;
+    if (cost < least) {
+      least = cost;
+      best = c.cfg;
+    }
+  }
+  return best;
+}
+
+}  // namespace rsint
+
 namespace rshost {
 
 thread_local std::string g_err;
@@ -317,23 +366,10 @@ float near_cap(int64_t n_lens, float m_max) {
   return n_lens > 0 ? m_max : 0.f;
 }
 
-// Measured on squares of 256^2 to 4096^2 rays, 100 to 60000 lenses, unit and Salpeter masses, us (128x8x512 at two
-// CTAs per SM / the shape taken):
-//   * few lenses: a CTA's start and its per-ray epilogue weigh more than its sums, and sixteen warps per SM hide
-//     them: 128x4x256 at four CTAs per SM (100 lenses x 1000^2: 60.3 / 50.9, x 4096^2: 746 / 553; 300 x 1000^2:
-//     102 / 87; at 1000 lenses level: 3078 / 3100 for 4096^2).
-//   * fewer than one small CTA per SM: the largest share of an SM decides, four rays per thread (300 x 256^2: 31.7 /
-//     23.6, 60000 x 256^2: 2215 / 1369).
-//   * else 128x8x512 at three CTAs per SM (1e4 x 1536^2: 4375 / 4316; Salpeter 3000 x 4096^2: 9625 / 9240; nowhere
-//     more than 2 % behind).
 int pick_cfg(const rs_field* f, int64_t n_rows, int64_t n0) {
   const int mass = f->dev.has_mass != rsdev::kUnitMass ? 1 : 0;
   if (g_cfg_set[mass]) return g_cfg[mass];
-  constexpr int64_t kFewLenses = 768;
-  // CTAs of four warps x four rays per thread
-  const int64_t small = ((n_rows + 3) / 4) * ((n0 + 127) / 128);
-  if (f->n_lens > 256 && small <= num_sms(f->device)) return rsint::kFewRaysCfg;
-  return f->n_lens < kFewLenses ? rsint::kFewLensesCfg : rsint::kManyLensesCfg;
+  return rsint::shape_by_size(mass != 0, (double)f->n_lens, n_rows, n0, num_sms(f->device));
 }
 
 int mass_mode(bool weighted, float m_max) {
@@ -394,6 +430,18 @@ int rs_unset_launch_config(int has_masses) {
 int rs_launch_config_is_set(int has_masses, int* is_set) {
   if (!is_set) return fail(RS_EINVAL, "is_set is NULL");
   *is_set = g_cfg_set[has_masses ? 1 : 0] ? 1 : 0;
+  return RS_OK;
+}
+
+int rs_launch_config_by_size(int has_masses, int64_t n_lens, int64_t n_rows, int64_t n0, int sms, int* block,
+                             int* rays_per_thread, int* lens_tile, int* min_ctas) {
+  if (n_lens < 0 || n_rows < 0 || n0 < 0 || sms < 1)
+    return fail(RS_EINVAL, "n_lens, n_rows and n0 must be >= 0 and sms >= 1");
+  const rsint::KernelCfg& k = rsint::kCfgs[rsint::shape_by_size(has_masses != 0, (double)n_lens, n_rows, n0, sms)];
+  if (block) *block = k.block;
+  if (rays_per_thread) *rays_per_thread = k.rpt;
+  if (lens_tile) *lens_tile = k.tile;
+  if (min_ctas) *min_ctas = k.min_ctas;
   return RS_OK;
 }
 

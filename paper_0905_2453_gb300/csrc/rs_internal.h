@@ -36,11 +36,9 @@ constexpr KernelCfg kCfgs[] = {RS_LAUNCH_SHAPES(RS_CFG_ENTRY)};
 #undef RS_CFG_ENTRY
 constexpr int kNumCfg = (int)(sizeof(kCfgs) / sizeof(kCfgs[0]));
 constexpr int kDefaultCfg = 8;  // 128 threads x 8 rays x 512-lens tiles, two CTAs per SM
-// Shapes taken by size when the caller set none (rshost::pick_cfg).
-constexpr int kFewRaysCfg = 7, kManyLensesCfg = 10, kFewLensesCfg = 11;
-static_assert(kCfgs[7].rpt == 4 && kCfgs[7].tile == 512 && kCfgs[10].min_ctas == 3 && kCfgs[10].tile == 512 &&
-                  kCfgs[11].rpt == 4 && kCfgs[11].min_ctas == 4,
-              "the shapes that pick_cfg's rule was measured with");
+// Shape of a call of n_rows x n0 rays through n_lens lenses where the caller set none: of the four shapes of
+// kShapeCosts (rs_api.cu) the one whose largest share of an SM takes the least time.
+int shape_by_size(bool masses, double n_lens, int64_t n_rows, int64_t n0, int sms);
 // Fields of kWideMass run one shape whatever is set: the default one.
 constexpr int kWideWarps = 4, kWideRpt = 8, kWideTile = 512;
 static_assert(kCfgs[kDefaultCfg].block == 32 * kWideWarps && kCfgs[kDefaultCfg].rpt == kWideRpt &&
