@@ -322,7 +322,8 @@ int rs_magnification(const uint32_t* d_counts, const rs_ray_grid* g, const rs_wi
  *   counts and out-of-window counters on every launch.
  * rs_batch_create_shaped -- as rs_batch_create with a launch shape per field: shapes = host int[4 *
  *   n_fields] of (block, rays per thread, lens tile, min_ctas) from rs_launch_configs (NULL: every field
- *   takes its mass mode's rs_set_launch_config shape, before one is set a shape by its lens count).  The items of each (shape, mass mode) form one
+ *   takes its mass mode's rs_set_launch_config shape; while none is set, a shape by its lenses and the
+ *   batch's work).  The items of each (shape, mass mode) form one
  *   persistent launch of the graph; the counts are the same bits for every choice.
  * rs_batch_launch -- replay the plan's graph on `stream`.
  * rs_batch_destroy -- release the plan (synchronises first).  NULL is a no-op.
@@ -360,14 +361,17 @@ int rs_field_status(rs_field_t f, int clear, int* status);
  * rs_set_launch_config selects the shape used by rs_shoot / rs_shoot_rows /
  * rs_shoot_rows_noalloc (and by batches planned afterwards) for fields without
  * (has_masses = 0) or with per-lens masses; RS_EINVAL for a shape that is not
- * compiled.  Until it is called for a mass mode, and again after rs_unset_launch_config, the
- * library takes a shape per call by the number of lenses and rays (batches: by the number of
- * lenses of each field); rs_get_launch_config then reports 128 x 8 x 512 at two CTAs per SM and
- * rs_launch_config_is_set reports 0 (1 once a shape was set): a caller that sets a shape for a
- * while puts back what was there with either of the two.  rs_launch_config_by_size reports the shape
- * so taken for n_rows x n0 rays through n_lens lenses on a device of sms SMs.  rs_launch_configs lists the compiled shapes: up to `cap`
- * (block, rpt, lens_tile, min_ctas) quadruples into `shapes` (int[4*cap]);
- * returns the number available via *count.  rs_launch_occupancy reports how
+ * compiled.  Until it is called for a mass mode, and again after
+ * rs_unset_launch_config, the library takes a shape per call by the number of
+ * lenses and rays (batches: by each field's lenses and the whole batch's work);
+ * rs_get_launch_config then reports 128 x 8 x 512 at two CTAs per SM and
+ * rs_launch_config_is_set reports 0 (1 once a shape was set): a caller that sets
+ * a shape for a while puts back what was there with either of the two.
+ * rs_launch_config_by_size reports the shape so taken for n_rows x n0 rays
+ * through n_lens lenses on a device of sms SMs.  rs_launch_configs lists the
+ * compiled shapes: up to `cap` (block, rpt, lens_tile, min_ctas) quadruples into
+ * `shapes` (int[4*cap]); returns the number available via *count.
+ * rs_launch_occupancy reports how
  * many CTAs of a shape's shoot kernel are resident per SM on the current device
  * (SMs x that = one wave of CTAs).
  */

@@ -117,6 +117,11 @@ namespace rsint {
 // large CTAs leave an SM's share uneven, us (two-CTA / chosen): 1e4 lenses x 288^2 394 / 376, x 640^2 1161 / 941,
 // x 8192 x 64 1164 / 1076, 6e4 x 512^2 3646 / 3646, 120 x 1000^2 64 / 54.  Three CTAs per SM whatever the share, as
 // below one large CTA per SM, is up to 7.5 % behind (2048 x 40 rays, 6e4 lenses).
+//
+// Persistent kernels (batches): the items left for a last round go to whichever CTAs finish first, three to an SM in
+// the three-CTA build, where the block scheduler would spread them.  5 fields of 2e4 lenses x 400^2 rays, 1000 large
+// items: 4473 us at three CTAs, 3876 at two; from a share of 8 on three are 0.9 to 4 % ahead in most sizes (8 fields
+// x 600^2, a share of 24: 1000 lenses 0.976, 3000 lenses 1.025).
 struct ShapeCost {
   int cfg;
   double lens[2][5];
@@ -133,7 +138,7 @@ static_assert(kCfgs[8].rpt == 8 && kCfgs[8].tile == 512 && kCfgs[8].min_ctas == 
                   kCfgs[7].min_ctas == 2 && kCfgs[11].rpt == 4 && kCfgs[11].tile == 256 && kCfgs[11].min_ctas == 4,
               "the shapes that kShapeCosts was measured with");
 
-int shape_by_size(bool masses, double n_lens, int64_t n_rows, int64_t n0, int sms) {
+int shape_by_size(bool masses, double n_lens, int64_t n_rows, int64_t n0, int sms, bool persistent) {
   int best = kDefaultCfg;
   double least = INFINITY;
   for (const ShapeCost& c : kShapeCosts) {
@@ -141,6 +146,7 @@ int shape_by_size(bool masses, double n_lens, int64_t n_rows, int64_t n0, int sm
     const int64_t warps = k.block / 32, seg = 32 * (int64_t)k.rpt;
     const double ctas = (double)((n_rows + warps - 1) / warps) * (double)((n0 + seg - 1) / seg);
     const double share = std::max(1.0, std::ceil(ctas / std::max(1, sms)));
+    if (persistent && k.min_ctas == 3 && share < 8.0) continue;
     const double* t = c.lens[masses ? 1 : 0];
     const double per_lens = share <= 4.0 ? t[(int)share - 1] : t[3] + (share - 4.0) * t[4];
     const double cost = per_lens * n_lens + c.cta * share;
@@ -366,10 +372,14 @@ float near_cap(int64_t n_lens, float m_max) {
   return n_lens > 0 ? m_max : 0.f;
 }
 
-int pick_cfg(const rs_field* f, int64_t n_rows, int64_t n0) {
+int pick_cfg(const rs_field* f, double n_lens, int64_t n_rows, int64_t n0, bool persistent) {
   const int mass = f->dev.has_mass != rsdev::kUnitMass ? 1 : 0;
   if (g_cfg_set[mass]) return g_cfg[mass];
-  return rsint::shape_by_size(mass != 0, (double)f->n_lens, n_rows, n0, num_sms(f->device));
+  return rsint::shape_by_size(mass != 0, n_lens, n_rows, n0, num_sms(f->device), persistent);
+}
+
+int pick_cfg(const rs_field* f, int64_t n_rows, int64_t n0) {
+  return pick_cfg(f, (double)f->n_lens, n_rows, n0, false);
 }
 
 int mass_mode(bool weighted, float m_max) {

@@ -31,6 +31,14 @@ struct rs_batch {
   cudaGraphExec_t exec;
 };
 
+namespace {
+
+// Per-ray cost of a field: one interaction per lens plus a fixed epilogue of about so many interactions.
+constexpr double kEpilogue = 64.0;
+double item_lenses(const rs_field* f) { return (double)f->n_lens + kEpilogue; }
+
+}  // namespace
+
 extern "C" {
 
 // ------------------------------------------------------------------------------------------------ batch
@@ -54,6 +62,8 @@ int rs_batch_create_shaped(int n_fields, const rs_field_t* fields, const rs_ray_
   constexpr int G = rs_batch::kGroups;
   std::vector<Item> items[G];
   int64_t n_total = 0;
+  double work = 0.0, work_lenses = 0.0, most = 0.0;  // in interactions: all fields, times their lenses, the largest
+  int64_t most_n0 = 1;
   for (int k = 0; k < n_fields; ++k) {
     if (!fields[k]) return fail(RS_EINVAL, "fields[%d] is NULL", k);
     if (fields[k]->device != dev) return fail(RS_EINVAL, "fields[%d] lives on another device", k);
@@ -63,9 +73,33 @@ int rs_batch_create_shaped(int n_fields, const rs_field_t* fields, const rs_ray_
     if ((rc = fill_desc(fields[k], &grids[k], 0, grids[k].n[1], &windows[k], d_counts[k],
                         d_out_of_window ? d_out_of_window + k : nullptr, &descs[k])) != RS_OK)
       return rc;
+    const double w = (double)descs[k].n_rows * (double)descs[k].n0 * item_lenses(fields[k]);
+    work += w;
+    work_lenses += w * (double)fields[k]->n_lens;
+    if (w > most) {
+      most = w;
+      most_n0 = descs[k].n0;
+    }
+  }
+  // without shapes of the caller's: the shape of a plain call of as many rays through a field as make the whole
+  // batch's work, since the fields share the SMs.  Two fields of 1000 lenses x 200^2 rays: 73 us by lens count alone, 61
+  // so.  Batches of less than kOneShape large CTAs per SM take one shape for all fields of a mass mode, by their mean
+  // lens count: a second group's CTAs wait for the first one's.  One shape / a shape per field, us, uneven fields of so
+  // many large CTAs per SM: 8.4 487 / 538, 15 (masses) 1314 / 1382, 17 591 / 552, 25 2769 / 2770, 36 1214 / 1212.
+  constexpr double kOneShape = 16.0;
+  const double mean_lenses = work > 0.0 ? work_lenses / work : 0.0;
+  const double mean_rays = work / (mean_lenses + kEpilogue);
+  const bool one_shape = mean_rays < kOneShape * 1024.0 * num_sms(dev);
+  for (int k = 0; k < n_fields; ++k) {
+    const int64_t n0 = descs[k].n0, nr = descs[k].n_rows;
     const int mass = fields[k]->dev.has_mass;
-    // without a shape of the caller's: by lens count only, as the other fields fill the chip
-    int cfg = pick_cfg(fields[k], (int64_t)1 << 20, (int64_t)1 << 10);
+    int cfg = rsint::kDefaultCfg;
+    if (!shapes && n0 > 0) {
+      const double lenses = one_shape ? mean_lenses : (double)fields[k]->n_lens;
+      const int64_t row = one_shape ? most_n0 : n0;
+      const double rows = std::ceil(work / (lenses + kEpilogue) / (double)row);
+      cfg = pick_cfg(fields[k], lenses, (int64_t)std::min(rows, 0x1p40), row, true);
+    }
     if (shapes) {
       const int* sh = shapes + 4 * k;
       cfg = rsint::find_cfg(sh[0], sh[1], sh[2], sh[3]);
@@ -77,7 +111,6 @@ int rs_batch_create_shaped(int n_fields, const rs_field_t* fields, const rs_ray_
     const int grp = rs_batch::kMassModes * cfg + mass;
     const int warps = rsint::kCfgs[cfg].block / 32;
     const int64_t seg = 32 * (int64_t)rsint::kCfgs[cfg].rpt;
-    const int64_t n0 = descs[k].n0, nr = descs[k].n_rows;
     if (n0 == 0 || nr == 0) continue;
     const int64_t ncol = (n0 + seg - 1) / seg;
     const int64_t nt = ((nr + warps - 1) / warps) * ncol;
@@ -87,8 +120,7 @@ int rs_batch_create_shaped(int n_fields, const rs_field_t* fields, const rs_ray_
       const int64_t trow = t / ncol, tcol = t - trow * ncol;
       const int64_t rows = std::min<int64_t>(warps, nr - trow * warps);
       const int64_t cols = std::min<int64_t>(seg, n0 - tcol * seg);
-      // per-ray cost: one interaction per lens plus a fixed epilogue (~ 64 interactions)
-      const double cost = (double)(rows * cols) * ((double)fields[k]->n_lens + 64.0);
+      const double cost = (double)(rows * cols) * item_lenses(fields[k]);
       items[grp].push_back({cost, k, (int)t});
     }
   }
@@ -107,7 +139,10 @@ int rs_batch_create_shaped(int n_fields, const rs_field_t* fields, const rs_ray_
     if (b->n_items[grp] == 0) continue;
     int bps = 0;
     if (rsint::batch_blocks_per_sm(grp / rs_batch::kMassModes, grp % rs_batch::kMassModes, &bps) != cudaSuccess || bps < 1) bps = 1;
-    b->grid[grp] = num_sms(dev) * bps;
+    // no more CTAs than items: the block scheduler spreads them over the SMs, where idle CTAs of one SM would race
+    // for two or three items each (one field of 3000 lenses x 300^2 rays, 150 items for 456 CTAs: 299 us with all of
+    // them, 153 so)
+    b->grid[grp] = std::min(num_sms(dev) * bps, b->n_items[grp]);
   }
   auto cleanup = [&]() {
     if (b->exec) cudaGraphExecDestroy(b->exec);

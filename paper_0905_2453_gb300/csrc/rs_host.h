@@ -34,6 +34,8 @@ namespace rshost {
 extern int g_cfg[2];
 // Shape of a call of n_rows x n0 rays through f: the caller's (rs_set_launch_config), or by size.
 int pick_cfg(const rs_field* f, int64_t n_rows, int64_t n0);
+// The same with the size given, and for the batch kernel (persistent).
+int pick_cfg(const rs_field* f, double n_lens, int64_t n_rows, int64_t n0, bool persistent);
 // Certified binning (float-float re-evaluation of rays inside their error band of a pixel edge).
 extern int g_certify;
 // Device memory for the per-ray state of a staged (lens-partitioned) shoot; larger calls run in row blocks.

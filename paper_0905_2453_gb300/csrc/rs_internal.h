@@ -38,7 +38,7 @@ constexpr int kNumCfg = (int)(sizeof(kCfgs) / sizeof(kCfgs[0]));
 constexpr int kDefaultCfg = 8;  // 128 threads x 8 rays x 512-lens tiles, two CTAs per SM
 // Shape of a call of n_rows x n0 rays through n_lens lenses where the caller set none: of the four shapes of
 // kShapeCosts (rs_api.cu) the one whose largest share of an SM takes the least time.
-int shape_by_size(bool masses, double n_lens, int64_t n_rows, int64_t n0, int sms);
+int shape_by_size(bool masses, double n_lens, int64_t n_rows, int64_t n0, int sms, bool persistent = false);
 // Fields of kWideMass run one shape whatever is set: the default one.
 constexpr int kWideWarps = 4, kWideRpt = 8, kWideTile = 512;
 static_assert(kCfgs[kDefaultCfg].block == 32 * kWideWarps && kCfgs[kDefaultCfg].rpt == kWideRpt &&

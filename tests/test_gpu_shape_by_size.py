@@ -65,3 +65,33 @@ def test_counts_do_not_depend_on_the_shape_taken(mass):
             f.close()
     if sms == 152:
         assert seen == {LARGE2, LARGE3, SMALL2, SMALL4}
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("fields", [[(1300, 200, "equal")], [(100, 300, "equal"), (5000, 150, "salpeter")],
+                                    [(100, 300, "salpeter"), (700, 260, "equal"), (900, 0, "equal"), (3000, 37, "equal")],
+                                    [(700, 300, "salpeter")] * 5])
+def test_batches_of_few_fields(fields):
+    """Batches whose items do not fill the SMs (fewer items than CTAs, a field without rays) give the plain counts."""
+    m = rs()
+    specs = [ri.disc_field("few", n, 0.5, 0.0, 0.2, side or 16, 48, seed=n + k, mass=mass)
+             for k, (n, side, mass) in enumerate(fields)]
+    grids = [s.grid if side else m.RayGrid(s.grid.origin, s.grid.spacing, (0, 5)) for s, (_, side, _) in zip(specs, fields)]
+    fs = [m.Field.from_spec(s) for s in specs]
+    try:
+        b = m.Batch(fs, grids, [s.window for s in specs])
+        try:
+            b.launch()
+            b.launch()  # the plan zeroes its counts
+            torch.cuda.synchronize()
+            for k, (f, s) in enumerate(zip(fs, specs)):
+                c = torch.zeros((48, 48), dtype=torch.int32, device="cuda")
+                o = torch.zeros(1, dtype=torch.int64, device="cuda")
+                if grids[k].n[0]:
+                    f.shoot(grids[k], s.window, c, o)
+                assert torch.equal(b.counts[k], c) and int(b.out_of_window[k].item()) == int(o.item()), k
+        finally:
+            b.close()
+    finally:
+        for f in fs:
+            f.close()
