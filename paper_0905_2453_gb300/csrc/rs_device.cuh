@@ -312,11 +312,11 @@ __device__ __forceinline__ void near_set_box(NS& ns, int g, float x1a, float x1b
 // The calling warp's share of the current tile (cnt lenses at l4, field index of the first: base):
 // lenses inside a group's box are appended to that group's list of parity par.  Whole warps call it.
 template <int TILE, class NS>
-__device__ __forceinline__ void near_gather(NS& ns, int par, const float4* l4, int cnt, int base, int nwarps) {
-  constexpr int NG = NS::kGroups;
+__device__ __forceinline__ void near_gather(NS& ns, int par, const float4* l4, int cnt, int base) {
+  constexpr int NG = NS::kGroups, WARPS = NS::kThreads * NG / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (NG > 1 && threadIdx.x == 0) ns.base[par] = base;
-  const int share = (TILE + nwarps - 1) / nwarps;
+  const int share = ((cnt + WARPS - 1) / WARPS + 31) / 32 * 32;  // whole turns of a warp
   const int l0 = warp * share, l1 = min(l0 + share, cnt);
   for (int l = l0 + lane; l - lane < l1; l += 32) {  // warp-uniform trip count
     const bool ok = l < l1;
@@ -719,6 +719,11 @@ __device__ __forceinline__ bool deflect_accumulate(const FieldDev& f, const uint
   static_assert(TILE % kGroup == 0 && kGroup % 8 == 0, "lens tile must hold whole lens groups");
   static_assert(kRenorm % kGroup == 0, "renormalisation falls on group boundaries");
   constexpr int NP = RPT / 2;
+  // Lens blocks of a group in line: all eight, but two in the cell kernel, whose sixteen near-lens boxes take 13 KB of
+  // code.  With eight it came to 134 KB (masses), and few lenses stream through all of it for every pass: ncu showed
+  // 3.9 warps per issue waiting for instructions (1.9 at 121 KB, before the boxes).  108 KB now; zoom of 341 masses
+  // on a grid of 11600^2 rays, 17.7e6 of them shot: 5.09 -> 3.62 ms, through 1e4 unit masses 4.25 -> 4.17 ms.
+  constexpr int kInLine = NS::kGroups > 1 ? 2 : kGroup / 8;
   const int n = f.n_lens;
   const int ntiles = (n + TILE - 1) / TILE;
   // the thread's first row of the CTA (shoot tiles: RayTile)
@@ -747,7 +752,7 @@ __device__ __forceinline__ bool deflect_accumulate(const FieldDev& f, const uint
       // the previous tile's list is complete (end-of-tile barrier); this tile's share goes to the other list
       if (t > 0) near_eval<NP, MASS>(*ns, (t - 1) & 1, (int)threadIdx.x / NS::kThreads, f, X1, X2,
                                      (int)blockDim.x);
-      near_gather<TILE>(*ns, t & 1, &sm.lens4[b][0], cnt, t * TILE, (int)(blockDim.x >> 5));
+      near_gather<TILE>(*ns, t & 1, &sm.lens4[b][0], cnt, t * TILE);
     }
     const uint32_t lbase = smem_u32(&sm.lens4[b][0]);
     const uint32_t xbase = smem_u32(&sm.x1tab[0]);
@@ -758,7 +763,7 @@ __device__ __forceinline__ bool deflect_accumulate(const FieldDev& f, const uint
         uint64_t P1[NP], P2[NP];
 #pragma unroll
         for (int q = 0; q < NP; ++q) P1[q] = P2[q] = 0ull;
-#pragma unroll
+#pragma unroll kInLine
         for (int p4 = 0; p4 < kGroup / 8; ++p4)
           lens_block<RPT, TILE, MASS, ROW>(lbase, xbase, mbase, rt, g + p4 * 8, X1, X2, P1, P2);
         fold_group<NP>(acc, P1, P2);
