@@ -852,7 +852,7 @@ int rs_shoot_culled(rs_field_t f, const rs_ray_grid* g, int64_t row_begin, int64
   e = cudaMemsetAsync(base, 0, 32, s);
   if (e == cudaSuccess)
     e = rsint::launch_cull(d, w->hi[0], w->hi[1], coarse, n_coarse_kept, mid, n_mid_kept, cells, n_kept,
-                           reinterpret_cast<unsigned long long*>(d_rays_shot), s);
+                           reinterpret_cast<unsigned long long*>(d_rays_shot), num_sms(f->device), s);
   if (e == cudaSuccess) {
     const int64_t want = (n_cells + 15) / 16;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms(f->device) * 2));

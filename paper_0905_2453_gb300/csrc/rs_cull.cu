@@ -17,6 +17,8 @@
 // x4 zoom of the 1e4-lens map, 4.12e6 rays in the window: 8.52e6 rays shot with cells of 16 x 16 and no linear term
 // (|alpha(x) - alpha(c)| <= rho sum m / (d (d - rho))), 6.78e6 with it -- most of the rest in cells a few rho from a
 // lens, whose area shrinks with the cell's -- hence the cells of 8 x 8.
+#include <algorithm>
+
 #include "rs_internal.h"
 
 namespace {
@@ -26,7 +28,8 @@ using namespace rsdev;
 constexpr int kCell = 8;         // rays per side of the cells that are shot
 constexpr int kMid = 16;         // of the second level
 constexpr int kCoarse = 64;      // and of the first
-constexpr int kCullBlock = 256;  // cells per CTA of the bound kernel
+constexpr int kCullBlock = 256;  // threads per CTA of the bound kernel
+constexpr int kCullSmThreads = 512;  // threads per SM up to which a cell's sums are shared
 
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
@@ -47,36 +50,50 @@ __device__ __forceinline__ void fold(float& hi, float& lo, float p) {
   hi = t;
 }
 
-// One thread per cell: the bound sums over all lenses (tiles staged in shared memory), then the
-// cell's source-plane box against the window.  Kept cells are appended to `out`; skipped cells add
+// Threads that share a cell's sums (a power of two up to a warp): as many as keep all cells' threads within `threads`,
+// so that a level of few cells still fills the chip, and leave each thread 64 lenses or more (each has the float64
+// bound of its cell to work out as well).  With one thread per cell a level takes as long as one thread's walk over
+// all lenses, however few its cells are: 30000 lenses, 500^2 rays 1.17 ms for each of the three levels, call 5.58 ->
+// 2.56 ms; 64 lenses a thread against none at 60 lenses, 3600^2 rays 94 against 160 us.
+__host__ __device__ __forceinline__ int cull_lanes(int64_t cells, int64_t threads, int n_lens) {
+  int lanes = 1;
+  while (lanes < 32 && cells * (2 * lanes) <= threads && n_lens >= 128 * lanes) lanes *= 2;
+  return lanes;
+}
+
+__device__ __forceinline__ double sum_over_lanes(double v, int lanes) {
+  for (int o = 1; o < lanes; o *= 2) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// cull_lanes threads per cell: the bound sums over all lenses (tiles staged in shared memory), then
+// the cell's source-plane box against the window.  Kept cells are appended to `out`; skipped cells add
 // their rays to the out-of-window count.  The first level takes every cell of the call (parent == nullptr), the
 // others the split x split cells of every kept cell of the level before.
 template <bool MASS>
 __global__ void __launch_bounds__(kCullBlock)
     cull_kernel(const ShootDesc d, int cell_rays, int64_t n_cx, int64_t n_cells, const unsigned* __restrict__ parent,
-                const unsigned* __restrict__ parent_count, int64_t n_px, int split, double hi0, double hi1,
-                unsigned* __restrict__ out, unsigned* __restrict__ out_count, unsigned long long* __restrict__ n_shot) {
+                const unsigned* __restrict__ parent_count, int64_t n_px, int split, int64_t threads, double hi0,
+                double hi1, unsigned* __restrict__ out, unsigned* __restrict__ out_count, unsigned long long* __restrict__ n_shot) {
   __shared__ float4 s_lens[kCullBlock];
   __shared__ float s_mass[kCullBlock];
   const int64_t n_cy = (d.n_rows + cell_rays - 1) / cell_rays;
+  const int children = split * split;
+  if (parent != nullptr) n_cells = (int64_t)*parent_count * children;
+  const int lanes = cull_lanes(n_cells, threads, d.f.n_lens);
+  if ((int64_t)blockIdx.x * kCullBlock >= n_cells * lanes) return;  // CTA-uniform: no cells left
+  const int64_t c = ((int64_t)blockIdx.x * kCullBlock + threadIdx.x) >> (__ffs(lanes) - 1);
+  const int share = (int)threadIdx.x & (lanes - 1);  // the thread takes lenses share, share + lanes, ...
   int64_t cx, cy;
-  bool ok;
+  bool ok = c < n_cells;
   if (parent != nullptr) {
-    const int64_t pc = *parent_count;
-    const int children = split * split;
-    if ((int64_t)blockIdx.x * kCullBlock >= pc * children) return;  // CTA-uniform: no parent cells left
-    const int64_t t = (int64_t)blockIdx.x * kCullBlock + threadIdx.x;
-    const int64_t slot = t / children;
-    const int sub = (int)(t % children);
-    ok = slot < pc;
-    const int64_t p = parent[ok ? slot : 0];
+    const int64_t p = parent[ok ? c / children : 0];
+    const int sub = (int)(c % children);
     const int64_t py = p / n_px, px = p - py * n_px;
     cx = px * split + sub % split;
     cy = py * split + sub / split;
     ok = ok && cx < n_cx && cy < n_cy;
   } else {
-    const int64_t c = (int64_t)blockIdx.x * kCullBlock + threadIdx.x;
-    ok = c < n_cells;
     cy = c / n_cx;
     cx = c - cy * n_cx;
   }
@@ -94,16 +111,22 @@ __global__ void __launch_bounds__(kCullBlock)
   float q1h = 0.f, q1l = 0.f, q2h = 0.f, q2l = 0.f;
   bool near = false;
   const int n = d.f.n_lens;
+  float4 next = make_float4(0.f, 0.f, 0.f, 0.f);  // the thread's lens of the tile after the one summed
+  float next_m = 0.f;
+  auto fetch = [&](int l) {
+    if (l >= n) return;
+    next = d.f.lens4[l];
+    if (MASS) next_m = d.f.mass2[l].x;
+  };
+  fetch((int)threadIdx.x);
   for (int t0 = 0; t0 < n; t0 += kCullBlock) {
     __syncthreads();
-    const int l = t0 + threadIdx.x;
-    if (l < n) {
-      s_lens[threadIdx.x] = d.f.lens4[l];
-      if (MASS) s_mass[threadIdx.x] = d.f.mass2[l].x;
-    }
+    s_lens[threadIdx.x] = next;
+    if (MASS) s_mass[threadIdx.x] = next_m;
     __syncthreads();
+    if (n - t0 > kCullBlock) fetch(t0 + kCullBlock + (int)threadIdx.x);
     const int cnt = min(kCullBlock, n - t0);
-    for (int g = 0; g < cnt; g += 32) {
+    for (int g = 0; g < cnt; g += 32 * lanes) {  // at most 32 terms of the thread
       float pa1 = 0.f, pa2 = 0.f, pb = 0.f, ps = 0.f, pq1 = 0.f, pq2 = 0.f;
       auto term = [&](int q) {
         const float4 L = s_lens[q];
@@ -128,11 +151,13 @@ __global__ void __launch_bounds__(kCullBlock)
         ps += mg;
         pb = fmaf(mg, r2, pb);
       };
-      if (g + 32 <= cnt) {
+      if (lanes == 1 && g + 32 <= cnt) {
 #pragma unroll 8
         for (int q = g; q < g + 32; ++q) term(q);
       } else {
-        for (int q = g; q < cnt; ++q) term(q);
+        const int end = min(g + 32 * lanes, cnt);
+#pragma unroll 4
+        for (int q = g + share; q < end; q += lanes) term(q);
       }
       fold(a1h, a1l, pa1);
       fold(a2h, a2l, pa2);
@@ -142,16 +167,22 @@ __global__ void __launch_bounds__(kCullBlock)
       fold(sh, sl, ps);
     }
   }
+  ok = ok && share == 0;  // one thread speaks for the cell
   const unsigned rays = ok ? (unsigned)((i1 - i0 + 1) * (r1 - r0 + 1)) : 0u;  // at most 64 x 64
   bool keep = true;
+  near = sum_over_lanes(near ? 1.0 : 0.0, lanes) > 0.0;
+  const double sum_s = sum_over_lanes((double)sh + (double)sl, lanes);
+  const double sum_b = sum_over_lanes((double)bh + (double)bl, lanes);
+  const double A1 = sum_over_lanes((double)a1h + (double)a1l, lanes);
+  const double A2 = sum_over_lanes((double)a2h + (double)a2l, lanes);
+  const double Q1 = sum_over_lanes((double)q1h + (double)q1l, lanes);
+  const double Q2 = 2.0 * sum_over_lanes((double)q2h + (double)q2l, lanes);
   if (!near) {
     // terms carry a few 2^-22 relative (approximate reciprocal square root and reciprocal, the gap's
     // cancellation when d is near 1.02 rho: <= 2^-15), sums of 32 float terms ~2^-19 of their
     // absolute sum: inflate B and S by 2^-8
-    const double S = ((double)sh + (double)sl) * (1.0 + 0x1p-8);
-    const double B = (double)rho * (double)rho * ((double)bh + (double)bl) * (1.0 + 0x1p-8);
-    const double A1 = (double)a1h + (double)a1l, A2 = (double)a2h + (double)a2l;
-    const double Q1 = (double)q1h + (double)q1l, Q2 = 2.0 * ((double)q2h + (double)q2l);
+    const double S = sum_s * (1.0 + 0x1p-8);
+    const double B = (double)rho * (double)rho * sum_b * (1.0 + 0x1p-8);
     // alpha(c) error <= ~2^-18.4 S, a ray's float32 error <= 72 u S = 2^-17.8 S, the linear term's error <= rho 2^-18
     // sum m / d^2 <= 2^-20 S per coefficient (rho (d - rho) <= d^2 / 4): together below 2^-16 S, taken twice; and
     // float64 roundings
@@ -261,28 +292,34 @@ int64_t cull_mid_cells(int64_t n_rows, int64_t n0) { return cells_of(n_rows, n0,
 template <bool MASS>
 static void launch_cull_m(const rsdev::ShootDesc& d, double hi0, double hi1, unsigned* coarse, unsigned* n_coarse,
                           unsigned* mid, unsigned* n_mid, unsigned* list, unsigned* n_kept, unsigned long long* n_shot,
-                          cudaStream_t s) {
+                          int sms, cudaStream_t s) {
   const auto across = [&](int side) { return (d.n0 + side - 1) / side; };
-  const auto blocks = [](int64_t cells) { return (unsigned)((cells + kCullBlock - 1) / kCullBlock); };
+  const int64_t threads = (int64_t)sms * kCullSmThreads;
+  // CTAs of a level of `cells` cells at most; where few cells are left, their lanes fill up to `threads`
+  const auto blocks = [&](int64_t cells) {
+    const int64_t t = std::max(cells, std::min(cells * cull_lanes(1, threads, d.f.n_lens), threads));
+    return (unsigned)((t + kCullBlock - 1) / kCullBlock);
+  };
   const int64_t n1 = cull_coarse_cells(d.n_rows, d.n0);
   constexpr int S2 = kCoarse / kMid, S3 = kMid / kCell;
   // the lower levels are launched for all cells the level above could keep; CTAs beyond what it kept leave at once
-  cull_kernel<MASS><<<blocks(n1), kCullBlock, 0, s>>>(d, kCoarse, across(kCoarse), n1, nullptr, nullptr, 0, 1, hi0, hi1,
-                                                      coarse, n_coarse, nullptr);
+  cull_kernel<MASS><<<blocks(n1), kCullBlock, 0, s>>>(d, kCoarse, across(kCoarse), n1, nullptr, nullptr, 0, 1, threads,
+                                                      hi0, hi1, coarse, n_coarse, nullptr);
   cull_kernel<MASS><<<blocks(n1 * S2 * S2), kCullBlock, 0, s>>>(d, kMid, across(kMid), 0, coarse, n_coarse,
-                                                                across(kCoarse), S2, hi0, hi1, mid, n_mid, nullptr);
+                                                                across(kCoarse), S2, threads, hi0, hi1, mid, n_mid,
+                                                                nullptr);
   cull_kernel<MASS><<<blocks(cull_mid_cells(d.n_rows, d.n0) * S3 * S3), kCullBlock, 0, s>>>(
-      d, kCell, across(kCell), 0, mid, n_mid, across(kMid), S3, hi0, hi1, list, n_kept, n_shot);
+      d, kCell, across(kCell), 0, mid, n_mid, across(kMid), S3, threads, hi0, hi1, list, n_kept, n_shot);
 }
 
 cudaError_t launch_cull(const rsdev::ShootDesc& d, double hi0, double hi1, unsigned* coarse, unsigned* n_coarse,
                         unsigned* mid, unsigned* n_mid, unsigned* list, unsigned* n_kept, unsigned long long* n_shot,
-                        cudaStream_t s) {
+                        int sms, cudaStream_t s) {
   if (cull_coarse_cells(d.n_rows, d.n0) <= 0) return cudaSuccess;
   if (d.f.has_mass)
-    launch_cull_m<true>(d, hi0, hi1, coarse, n_coarse, mid, n_mid, list, n_kept, n_shot, s);
+    launch_cull_m<true>(d, hi0, hi1, coarse, n_coarse, mid, n_mid, list, n_kept, n_shot, sms, s);
   else
-    launch_cull_m<false>(d, hi0, hi1, coarse, n_coarse, mid, n_mid, list, n_kept, n_shot, s);
+    launch_cull_m<false>(d, hi0, hi1, coarse, n_coarse, mid, n_mid, list, n_kept, n_shot, sms, s);
   return cudaGetLastError();
 }
 

@@ -123,7 +123,7 @@ int64_t cull_mid_cells(int64_t n_rows, int64_t n0);
 int64_t cull_coarse_cells(int64_t n_rows, int64_t n0);
 cudaError_t launch_cull(const rsdev::ShootDesc& d, double hi0, double hi1, unsigned* coarse, unsigned* n_coarse,
                         unsigned* mid, unsigned* n_mid, unsigned* list, unsigned* n_kept, unsigned long long* n_shot,
-                        cudaStream_t s);
+                        int sms, cudaStream_t s);
 cudaError_t launch_shoot_cells(const rsdev::ShootDesc& d, int64_t n_cx, const unsigned* list, const unsigned* n_kept,
                                int grid, cudaStream_t s);
 

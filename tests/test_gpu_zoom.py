@@ -100,3 +100,13 @@ def test_n1e4_culled_equals_plain():
     """The 1e4-lens workload: full-map culled shooting equals the plain shoot bit for bit."""
     frac = _same_as_plain(ri.n1e4_field())
     assert frac < 0.9
+
+
+@pytest.mark.parametrize("n", [127, 128, 1000, 5000])
+@pytest.mark.parametrize("side", [16, 65, 300])
+def test_few_cells_share_their_sums(n, side):
+    """Levels of few cells through many lenses split a cell's sums over up to 32 threads."""
+    spec = ri.disc_field("lanes", n, 0.5, 0.05, 0.2, side, 64, seed=n + side, mass="salpeter" if n & 1 else "equal")
+    _same_as_plain(spec)
+    lo, hi = np.asarray(spec.window.lo), np.asarray(spec.window.hi)
+    _same_as_plain(spec, window=ri.Window(tuple(lo + 0.4 * (hi - lo)), tuple(lo + 0.7 * (hi - lo)), (64, 64)))
