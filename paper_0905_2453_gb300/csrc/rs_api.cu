@@ -824,8 +824,7 @@ int rs_shoot_culled(rs_field_t f, const rs_ray_grid* g, int64_t row_begin, int64
   if ((rc = fill_desc(f, g, row_begin, row_end, w, d_counts, d_out_of_window, &d)) != RS_OK) return rc;
   if (d.n_rows == 0 || d.n0 == 0) return RS_OK;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  int64_t n_cx = 0;
-  const int64_t n_cells = rsint::cull_cells(d.n_rows, d.n0, &n_cx);
+  const int64_t n_cells = rsint::cull_cells(d.n_rows, d.n0);
   const int64_t n_coarse = rsint::cull_coarse_cells(d.n_rows, d.n0);
   const int64_t n_mid = rsint::cull_mid_cells(d.n_rows, d.n0);
   // stream-ordered workspace: [re-evaluation count | coarse count | mid count | kept count | re-evaluation list |
@@ -834,8 +833,25 @@ int rs_shoot_culled(rs_field_t f, const rs_ray_grid* g, int64_t row_begin, int64
   const size_t coarse_off = 32 + sizeof(uint2) * (size_t)cap;
   const size_t mid_off = coarse_off + sizeof(unsigned) * (size_t)n_coarse;
   const size_t list_off = mid_off + sizeof(unsigned) * (size_t)n_mid;
+  const size_t full = list_off + sizeof(unsigned) * (size_t)n_cells;
+  // The last list is four times the mid list (268 MB for 2^32 rays).  Where it cannot be had the kept 16 x 16 cells are
+  // shot as they are (a third more rays, the same counts), as they are while the stream is being captured, when a
+  // graph that cannot be given its memory fails only later.  Sizes compare in the allocator's granules: a call
+  // without a granule to save has nothing to fall back to.
+  const auto granules = [](size_t bytes) { return (bytes + ((size_t)2 << 20) - 1) >> 21; };
+  const bool saves = granules(full) > granules(list_off);
+  bool mid_cells = false;
+  if (saves) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    mid_cells = cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone;
+  }
   void* ws = nullptr;
-  cudaError_t e = dev_alloc_async(&ws, list_off + sizeof(unsigned) * (size_t)n_cells, s);
+  cudaError_t e = dev_alloc_async(&ws, mid_cells ? list_off : full, s);
+  if (e == cudaErrorMemoryAllocation && saves && !mid_cells) {
+    (void)cudaGetLastError();
+    mid_cells = true;
+    e = dev_alloc_async(&ws, list_off, s);
+  }
   if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (culled-shoot workspace)");
   char* base = reinterpret_cast<char*>(ws);
   unsigned* n_coarse_kept = reinterpret_cast<unsigned*>(base + 8);
@@ -843,7 +859,7 @@ int rs_shoot_culled(rs_field_t f, const rs_ray_grid* g, int64_t row_begin, int64
   unsigned* n_kept = reinterpret_cast<unsigned*>(base + 24);
   unsigned* coarse = reinterpret_cast<unsigned*>(base + coarse_off);
   unsigned* mid = reinterpret_cast<unsigned*>(base + mid_off);
-  unsigned* cells = reinterpret_cast<unsigned*>(base + list_off);
+  unsigned* cells = mid_cells ? nullptr : reinterpret_cast<unsigned*>(base + list_off);
   if (g_certify) {
     d.rc_cap = cap;
     d.rc_count = reinterpret_cast<unsigned int*>(base);
@@ -854,9 +870,9 @@ int rs_shoot_culled(rs_field_t f, const rs_ray_grid* g, int64_t row_begin, int64
     e = rsint::launch_cull(d, w->hi[0], w->hi[1], coarse, n_coarse_kept, mid, n_mid_kept, cells, n_kept,
                            reinterpret_cast<unsigned long long*>(d_rays_shot), num_sms(f->device), s);
   if (e == cudaSuccess) {
-    const int64_t want = (n_cells + 15) / 16;
+    const int64_t want = (n_cells + 15) / 16;  // sixteen 8 x 8 cells a CTA and pass
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms(f->device) * 2));
-    e = rsint::launch_shoot_cells(d, n_cx, cells, n_kept, grid, s);
+    e = rsint::launch_shoot_cells(d, mid_cells, mid_cells ? mid : cells, mid_cells ? n_mid_kept : n_kept, grid, s);
   }
   if (e == cudaSuccess && g_certify)
     e = rsint::launch_recheck(&d, nullptr, d.rc_list, d.rc_count, d.rc_cap, recheck_grid(f->device), s);

@@ -212,10 +212,11 @@ __global__ void __launch_bounds__(kCullBlock)
 }
 
 // Kept cells: a CTA of four warps shoots sixteen cells per pass; eight lanes share a cell, lane l of them holding
-// its row l (eight columns).  The per-ray arithmetic is rs_shoot's (per-ray squared distances instead of the shared
+// its row l (eight columns).  The list holds cells of 8 x 8, or (n_mx > 0, cells per row) of 16 x 16, whose four
+// children are then all shot.  The per-ray arithmetic is rs_shoot's (per-ray squared distances instead of the shared
 // row table give bitwise the same values).
 template <int MASS>
-__global__ void __launch_bounds__(128, 2) shoot_cells_kernel(const ShootDesc d, int64_t n_cx,
+__global__ void __launch_bounds__(128, 2) shoot_cells_kernel(const ShootDesc d, int64_t n_cx, int64_t n_mx,
                                                              const unsigned* __restrict__ list,
                                                              const unsigned* __restrict__ n_kept) {
   constexpr int RPT = kCell, CELLS = 128 / kCell;
@@ -223,13 +224,29 @@ __global__ void __launch_bounds__(128, 2) shoot_cells_kernel(const ShootDesc d, 
   __shared__ NearSmem<rsint::kTile, CELLS, 128, RPT> ns;  // one near-lens box per cell
   PipeState ps;
   pipe_init(sm.bar, ps);
-  const unsigned count = *n_kept;
+  constexpr unsigned CHILDREN = (kMid / kCell) * (kMid / kCell);
+  const unsigned count = *n_kept * (n_mx > 0 ? CHILDREN : 1u);
   const int lane = threadIdx.x & 31, own = threadIdx.x / kCell, row = threadIdx.x % kCell;
   for (unsigned base = blockIdx.x * (unsigned)CELLS; base < count; base += gridDim.x * (unsigned)CELLS) {  // CTA-uniform
     const unsigned slot = base + (unsigned)own;
-    const bool cell_ok = slot < count;
-    const int64_t cell = (int64_t)list[cell_ok ? slot : count - 1];
-    const int64_t cy = cell / n_cx, cx = cell - cy * n_cx;
+    bool cell_ok = slot < count;
+    const unsigned at = cell_ok ? slot : count - 1;
+    int64_t cx, cy;
+    if (n_mx > 0) {
+      const int64_t mid = (int64_t)list[at / CHILDREN];
+      const int64_t my = mid / n_mx, mx = mid - my * n_mx;
+      cx = mx * 2 + (at & 1u);
+      cy = my * 2 + ((at >> 1) & 1u);
+      if (cx >= n_cx || cy * kCell >= d.n_rows) {  // past the last column or row: no rays
+        cell_ok = false;
+        cx = mx * 2;
+        cy = my * 2;
+      }
+    } else {
+      const int64_t cell = (int64_t)list[at];
+      cy = cell / n_cx;
+      cx = cell - cy * n_cx;
+    }
     const int64_t jrel = cy * kCell + row;
     const bool row_ok = cell_ok && jrel < d.n_rows;
     const int64_t j = d.j_begin + (jrel < d.n_rows ? jrel : d.n_rows - 1);
@@ -278,14 +295,10 @@ __global__ void __launch_bounds__(128, 2) shoot_cells_kernel(const ShootDesc d, 
 
 namespace rsint {
 
-int64_t cull_cells(int64_t n_rows, int64_t n0, int64_t* n_cx) {
-  *n_cx = (n0 + kCell - 1) / kCell;
-  return ((n_rows + kCell - 1) / kCell) * *n_cx;
-}
-
 static int64_t cells_of(int64_t n_rows, int64_t n0, int side) {
   return ((n_rows + side - 1) / side) * ((n0 + side - 1) / side);
 }
+int64_t cull_cells(int64_t n_rows, int64_t n0) { return cells_of(n_rows, n0, kCell); }
 int64_t cull_coarse_cells(int64_t n_rows, int64_t n0) { return cells_of(n_rows, n0, kCoarse); }
 int64_t cull_mid_cells(int64_t n_rows, int64_t n0) { return cells_of(n_rows, n0, kMid); }
 
@@ -307,7 +320,8 @@ static void launch_cull_m(const rsdev::ShootDesc& d, double hi0, double hi1, uns
                                                       hi0, hi1, coarse, n_coarse, nullptr);
   cull_kernel<MASS><<<blocks(n1 * S2 * S2), kCullBlock, 0, s>>>(d, kMid, across(kMid), 0, coarse, n_coarse,
                                                                 across(kCoarse), S2, threads, hi0, hi1, mid, n_mid,
-                                                                nullptr);
+                                                                list ? nullptr : n_shot);
+  if (list == nullptr) return;
   cull_kernel<MASS><<<blocks(cull_mid_cells(d.n_rows, d.n0) * S3 * S3), kCullBlock, 0, s>>>(
       d, kCell, across(kCell), 0, mid, n_mid, across(kMid), S3, threads, hi0, hi1, list, n_kept, n_shot);
 }
@@ -323,14 +337,15 @@ cudaError_t launch_cull(const rsdev::ShootDesc& d, double hi0, double hi1, unsig
   return cudaGetLastError();
 }
 
-cudaError_t launch_shoot_cells(const rsdev::ShootDesc& d, int64_t n_cx, const unsigned* list, const unsigned* n_kept,
+cudaError_t launch_shoot_cells(const rsdev::ShootDesc& d, bool mid_cells, const unsigned* list, const unsigned* n_kept,
                                int grid, cudaStream_t s) {
+  const int64_t n_cx = (d.n0 + kCell - 1) / kCell, n_mx = mid_cells ? (d.n0 + kMid - 1) / kMid : 0;
   if (d.f.has_mass == rsdev::kWideMass)
-    shoot_cells_kernel<rsdev::kWideMass><<<grid, 128, 0, s>>>(d, n_cx, list, n_kept);
+    shoot_cells_kernel<rsdev::kWideMass><<<grid, 128, 0, s>>>(d, n_cx, n_mx, list, n_kept);
   else if (d.f.has_mass)
-    shoot_cells_kernel<rsdev::kMass><<<grid, 128, 0, s>>>(d, n_cx, list, n_kept);
+    shoot_cells_kernel<rsdev::kMass><<<grid, 128, 0, s>>>(d, n_cx, n_mx, list, n_kept);
   else
-    shoot_cells_kernel<rsdev::kUnitMass><<<grid, 128, 0, s>>>(d, n_cx, list, n_kept);
+    shoot_cells_kernel<rsdev::kUnitMass><<<grid, 128, 0, s>>>(d, n_cx, n_mx, list, n_kept);
   return cudaGetLastError();
 }
 

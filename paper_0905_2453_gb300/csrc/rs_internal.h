@@ -113,18 +113,19 @@ cudaError_t launch_batch(int cfg, int mass, const rsdev::ShootDesc* descs, const
 cudaError_t batch_blocks_per_sm(int cfg, int mass, int* blocks);
 
 // Culled shooting (rs_cull.cu): cells of 8 x 8 rays, bounded first in cells of 64 x 64 and 16 x 16.
-// cull_cells returns the number of 8 x 8 cells of a call (and the cells per row), cull_mid_cells and
-// cull_coarse_cells those of the levels above; launch_cull appends the 64 x 64 cells that may reach the window to
-// `coarse` (count *n_coarse), the 16 x 16 cells of those that may to `mid` and the 8 x 8 cells of these to `list`
-// (count *n_kept, rays in *n_shot if not null), counting the rays of all others out of window; launch_shoot_cells
-// shoots the listed cells (grid: persistent CTAs of 128 threads).  Counters start at zero.
-int64_t cull_cells(int64_t n_rows, int64_t n0, int64_t* n_cx);
+// cull_cells, cull_mid_cells and cull_coarse_cells return the number of 8 x 8, 16 x 16 and 64 x 64 cells of a call;
+// launch_cull appends the 64 x 64 cells that may reach the window to `coarse` (count *n_coarse), the 16 x 16 cells of
+// those that may to `mid` and the 8 x 8 cells of these to `list` (count *n_kept), counting the rays of all others out
+// of window (and those left in *n_shot if not null); with `list` null it stops at `mid`.  launch_shoot_cells
+// shoots the listed 8 x 8 cells, or 16 x 16 cells (mid_cells; grid: persistent CTAs of 128 threads).  Counters start
+// at zero.
+int64_t cull_cells(int64_t n_rows, int64_t n0);
 int64_t cull_mid_cells(int64_t n_rows, int64_t n0);
 int64_t cull_coarse_cells(int64_t n_rows, int64_t n0);
 cudaError_t launch_cull(const rsdev::ShootDesc& d, double hi0, double hi1, unsigned* coarse, unsigned* n_coarse,
                         unsigned* mid, unsigned* n_mid, unsigned* list, unsigned* n_kept, unsigned long long* n_shot,
                         int sms, cudaStream_t s);
-cudaError_t launch_shoot_cells(const rsdev::ShootDesc& d, int64_t n_cx, const unsigned* list, const unsigned* n_kept,
+cudaError_t launch_shoot_cells(const rsdev::ShootDesc& d, bool mid_cells, const unsigned* list, const unsigned* n_kept,
                                int grid, cudaStream_t s);
 
 // Lens-partitioned shooting (rs_staged.cu), default launch shape (4 warps x 8 rays): the per-ray

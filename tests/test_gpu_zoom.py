@@ -102,6 +102,49 @@ def test_n1e4_culled_equals_plain():
     assert frac < 0.9
 
 
+@pytest.mark.parametrize("n,mass", [(70, "equal"), (700, "salpeter")])
+def test_large_call_without_room_for_the_cell_list(n, mass):
+    """A call whose 8 x 8 cell list cannot be allocated, or whose stream is being captured, shoots its 16 x 16 cells:
+    the same counts, in the memory of the two upper lists.  (6007 x 6013 rays: neither side a multiple of a cell.)"""
+    m = rs()
+    spec = ri.disc_field("room", n, 0.5, 0.1, 0.3, 512, 96, seed=8, mass=mass)
+    g = spec.grid
+    fine = ri.RayGrid(g.origin, tuple(g.spacing[k] * 512 / q for k, q in ((0, 6007), (1, 6013))), (6007, 6013))
+    f = m.Field.from_spec(spec)
+    try:
+        def run(call):
+            c = torch.zeros((96, 96), dtype=torch.int32, device=dev())
+            o, shot = (torch.zeros(1, dtype=torch.int64, device=dev()) for _ in range(2))
+            call(c, o, shot)
+            torch.cuda.synchronize()
+            return c.cpu().numpy(), int(o.item()), int(shot.item())
+
+        culled = lambda c, o, shot: m.rs_shoot_culled(f.handle, fine, 0, 6013, spec.window, c, o, shot)  # noqa: E731
+
+        def refused(c, o, shot):
+            m.rs_set_alloc_failure(0)
+            try:
+                culled(c, o, shot)
+            finally:
+                m.rs_set_alloc_failure(-1)
+
+        def captured(c, o, shot):
+            graph = torch.cuda.CUDAGraph()
+            st = torch.cuda.Stream()
+            with torch.cuda.graph(graph, stream=st):
+                m.rs_shoot_culled(f.handle, fine, 0, 6013, spec.window, c, o, shot, stream=st)
+            graph.replay()
+
+        ref = run(lambda c, o, shot: m.rs_shoot(f.handle, fine, spec.window, c, o))
+        full, small, graph = run(culled), run(refused), run(captured)
+        for got in (full, small, graph):
+            assert np.array_equal(got[0], ref[0]) and got[1] == ref[1]
+        assert full[2] < small[2] == graph[2] < 6007 * 6013
+        assert f.status() == m.RS_OK
+    finally:
+        f.close()
+
+
 @pytest.mark.parametrize("n", [127, 128, 1000, 5000])
 @pytest.mark.parametrize("side", [16, 65, 300])
 def test_few_cells_share_their_sums(n, side):
