@@ -182,14 +182,22 @@ bool inject_alloc_failure() {
   return false;
 }
 
-constexpr int kPoolDevices = 64;
+// One pool per context that allocated (a device may have several; a device reset ends its contexts and their pools).
 struct Pool {
-  cudaMemPool_t pool = nullptr;
-  unsigned long long ctx = 0;  // id of the context the pool belongs to (a device reset ends it)
-  int fields = 0;              // live fields of the device
+  int device;
+  unsigned long long ctx;  // id of the context
+  cudaMemPool_t pool;      // nullptr: none could be made, the device's default one serves
+  int fields;              // live fields created under the context
 };
+constexpr size_t kMaxPools = 64;  // contexts of a process's life beyond this number take the device's default pool
 static std::mutex g_pool_mutex;
-static Pool g_pools[kPoolDevices];
+static std::vector<Pool>& g_pools = *new std::vector<Pool>();  // never destroyed: fields may outlive static objects
+
+static Pool* find_pool(int device, unsigned long long ctx) {
+  for (Pool& q : g_pools)
+    if (q.device == device && q.ctx == ctx) return &q;
+  return nullptr;
+}
 
 // Id of the current CUDA context, unique over the process's life (through the driver entry point, so the library
 // needs no link to the driver library); 0 where it cannot be queried.
@@ -208,47 +216,56 @@ static unsigned long long context_id() {
   return id;
 }
 
+// The entry of the current context, made on its first call (nullptr: kMaxPools reached).
+static Pool* pool_entry(int device, unsigned long long ctx) {
+  Pool* q = find_pool(device, ctx);
+  if (q != nullptr || g_pools.size() >= kMaxPools) return q;
+  g_pools.push_back(Pool{device, ctx, nullptr, 0});
+  return &g_pools.back();
+}
+
 cudaError_t pool_alloc_async(void** p, size_t bytes, cudaStream_t s) {
   int dev = -1;
   cudaMemPool_t pool = nullptr;
-  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kPoolDevices) {
-    const unsigned long long ctx = context_id();
+  const unsigned long long ctx = cudaGetDevice(&dev) == cudaSuccess ? context_id() : 0;
+  if (ctx != 0) {
     std::lock_guard<std::mutex> lock(g_pool_mutex);
-    Pool& q = g_pools[dev];
-    if (ctx != 0 && (q.pool == nullptr || q.ctx != ctx)) {
-      cudaMemPoolProps props = {};
-      props.allocType = cudaMemAllocationTypePinned;
-      props.location.type = cudaMemLocationTypeDevice;
-      props.location.id = dev;
-      uint64_t keep = kPoolKeep;
-      cudaMemPool_t made = nullptr;
-      if (cudaMemPoolCreate(&made, &props) == cudaSuccess &&
-          cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess) {
-        q.pool = made;
-        q.ctx = ctx;
-      } else if (made) {
-        cudaMemPoolDestroy(made);
+    if (Pool* q = pool_entry(dev, ctx)) {
+      if (q->pool == nullptr) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        uint64_t keep = kPoolKeep;
+        cudaMemPool_t made = nullptr;
+        if (cudaMemPoolCreate(&made, &props) == cudaSuccess &&
+            cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+          q->pool = made;
+        else if (made)
+          cudaMemPoolDestroy(made);
       }
+      pool = q->pool;
     }
-    if (q.pool != nullptr && q.ctx == ctx) pool = q.pool;
   }
   if (pool != nullptr) return cudaMallocFromPoolAsync(p, bytes, pool, s);
   (void)cudaGetLastError();
   return cudaMallocAsync(p, bytes, s);  // no pool of our own to be had: the device's default one
 }
 
-void pool_field_created(int device) {
-  if (device < 0 || device >= kPoolDevices) return;
+unsigned long long pool_field_created(int device) {
+  const unsigned long long ctx = context_id();
+  if (ctx == 0) return 0;
   std::lock_guard<std::mutex> lock(g_pool_mutex);
-  ++g_pools[device].fields;
+  if (Pool* q = pool_entry(device, ctx)) ++q->fields;
+  return ctx;
 }
 
-void pool_field_destroyed(int device) {
-  if (device < 0 || device >= kPoolDevices) return;
-  const unsigned long long ctx = context_id();
+void pool_field_destroyed(int device, unsigned long long ctx) {
+  if (ctx == 0) return;
+  const bool current = context_id() == ctx;  // a context that is not current may be gone, and its pool with it
   std::lock_guard<std::mutex> lock(g_pool_mutex);
-  Pool& q = g_pools[device];
-  if (--q.fields == 0 && q.pool != nullptr && q.ctx == ctx) cudaMemPoolTrimTo(q.pool, 0);
+  Pool* q = find_pool(device, ctx);
+  if (q != nullptr && --q->fields == 0 && q->pool != nullptr && current) cudaMemPoolTrimTo(q->pool, 0);
 }
 
 int recheck_grid(int device) {
@@ -610,7 +627,7 @@ int rs_create_field(const float* lens_xy, const float* masses, int64_t n_lens, d
   f->dev.lamabs = std::nextafter((float)std::max(std::fabs(f->dev.lam1), std::fabs(f->dev.lam2)), INFINITY);
   f->dev.mcap = near_cap(n_lens, f->dev.has_mass ? m_max : 1.f);
   f->dev.status = f->status;
-  pool_field_created(f->device);
+  f->pool_ctx = pool_field_created(f->device);
   *out = f;
   return RS_OK;
 }
@@ -625,7 +642,7 @@ int rs_destroy_field(rs_field_t f) {
   cudaFree(f->status);
   cudaFree(f->motion);
   if (f->parent) --f->parent->views;
-  pool_field_destroyed(f->device);
+  pool_field_destroyed(f->device, f->pool_ctx);
   delete f;
   return RS_OK;
 }
@@ -669,7 +686,7 @@ int rs_create_field_view(rs_field_t parent, int64_t lens_begin, int64_t n_lens, 
   f->dev.status = f->status;
   f->parent = parent;
   ++parent->views;
-  pool_field_created(f->device);
+  f->pool_ctx = pool_field_created(f->device);
   *out = f;
   return RS_OK;
 }

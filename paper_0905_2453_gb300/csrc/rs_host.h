@@ -26,6 +26,7 @@ struct rs_field {
   // of live views of a field (it cannot be destroyed while any is left)
   rs_field* parent = nullptr;
   int views = 0;
+  unsigned long long pool_ctx = 0;  // id of the context whose pool counts the field (0: none)
 };
 
 namespace rshost {
@@ -55,14 +56,14 @@ cudaError_t dev_alloc(T** p, size_t bytes) {
 }
 
 // Stream-ordered workspaces (released with cudaFreeAsync) come from a memory pool of the library's own, one per
-// device, that keeps up to kPoolKeep bytes across synchronisations.  The device's default pool gives everything
+// context, that keeps up to kPoolKeep bytes across synchronisations.  The device's default pool gives everything
 // back whenever the device is synchronised, and mapping a call's few hundred KiB again cost ~0.23 ms: a 384^2-ray
 // map through 300 lenses took 294 us alone against 60 us among others.  The pool is trimmed when the last field of
-// its device is destroyed; its allocator orders reuse across streams and threads.
+// its context is destroyed; its allocator orders reuse across streams and threads.
 constexpr uint64_t kPoolKeep = (uint64_t)128 << 20;
 cudaError_t pool_alloc_async(void** p, size_t bytes, cudaStream_t s);
-void pool_field_created(int device);
-void pool_field_destroyed(int device);  // device current and synchronised
+unsigned long long pool_field_created(int device);  // id of the current context
+void pool_field_destroyed(int device, unsigned long long ctx);  // device current and synchronised
 
 template <class T>
 cudaError_t dev_alloc_async(T** p, size_t bytes, cudaStream_t s) {
