@@ -264,7 +264,7 @@ int rs_partition_recheck(rs_field_t part, int weighted, const rs_ray_grid* g, in
  *              around y inside which the float32 result cannot decide a pixel (see
  *              certified binning below); asking for it costs one more pass over the lenses.
  * The per-ray arithmetic is the one rs_shoot uses, bit for bit (the band included).  Few rays
- * through many lenses take a stream-ordered workspace (at most 32 MiB + 36 bytes per ray) to sum a
+ * through many lenses take a stream-ordered workspace (at most 35 MiB) to sum a
  * ray's lens groups side by side; where it cannot be had, and while the stream is being captured,
  * the call runs without it, slower and with the same bits.
  */

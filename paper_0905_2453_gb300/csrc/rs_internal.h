@@ -76,14 +76,21 @@ cudaError_t shoot_blocks_per_sm(int cfg, bool mass, int* blocks);
 cudaError_t launch_trace(const rsdev::FieldDev& f, double or0, double or1, double sp0, double sp1,
                          const int64_t* ij, int64_t k, double* y, double* alpha, double* err, cudaStream_t s);
 
-// The same with the lens groups of every ray summed side by side (rs_trace.cu): ws holds trace_split_bytes, which
-// the workspace bound kTraceSplitBytes keeps below 32 MiB + 36 bytes per ray.  It pays where the direct kernel
-// (one thread per four rays over all lenses) leaves SMs idle or runs long serial loops; measured alone, us,
-// direct / split without | with error bands: 512 lenses x 1000 rays 54 / 67 | 115 / 82, 2000 x 4096 95 / 75 |
-// 318 / 84, 2000 x 65536 96 / 108 | 323 / 168, 20000 x 30000 596 / 300 | 4828 / 475, 1e6 x 10 27475 / 915.
+// The same with the lens groups of every ray summed side by side (rs_trace.cu): ws holds trace_split_bytes, at most
+// kTraceSplitBytes and 36 bytes per ray of a block (whole blocks of 128 rays, at most kTraceSplitRays: 34.25 MiB).
 constexpr size_t kTraceSplitBytes = (size_t)32 << 20;
+constexpr int64_t kTraceSplitRays = 65536;  // more rays run in blocks of so many
+// It pays where the direct kernel (one thread per four rays over all lenses) leaves SMs idle or, with error bands,
+// runs its second loop over all lenses with few warps; it costs more launches (46 us of host time a call against 35)
+// and more work per ray.  Device us, direct / split: without bands 1024 lenses x 32768 rays 31 / 27, 1536 43 / 32,
+// 2048 x 65536 56 / 56, 1e4 x 150000 401 / 542.  With bands 512 x 500 68 / 39 (100 rays, whole calls 46 / 48),
+// 1024 x 65536 133 / 69, and for more than a block of rays, which the direct kernel runs the better the more there
+// are: 1024 x 100000 148 / 114, 150000 150 / 176; 3000 x 200000 479 / 461; 5000 x 400000 1620 / 1382, 1e6 2881 / 3412;
+// 1e4 x 1e6 7375 / 5581.
 inline bool trace_split_pays(int n_lens, int64_t k, bool err) {
-  return err ? n_lens >= 512 && k <= 65536 : n_lens >= 1024 && k <= 32768;
+  if (!err) return n_lens >= 1536 && k <= 32768;
+  if (k <= kTraceSplitRays) return n_lens >= (k < 512 ? 640 : 512);
+  return n_lens >= 640 * ((k + kTraceSplitRays - 1) / kTraceSplitRays);
 }
 size_t trace_split_bytes(int n_lens, int64_t k);
 cudaError_t launch_trace_split(const rsdev::FieldDev& f, double or0, double or1, double sp0, double sp1,

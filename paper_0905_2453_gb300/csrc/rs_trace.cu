@@ -298,13 +298,15 @@ int64_t trace_chunk_groups(int64_t n_rb, int64_t n_groups) {
 }
 
 size_t trace_split_bytes(int n_lens, int64_t k) {
-  const int64_t n_rb = (k + kRb - 1) / kRb, n_groups = ((int64_t)n_lens + kGroup - 1) / kGroup;
+  const int64_t n_rb = (std::min(k, kTraceSplitRays) + kRb - 1) / kRb;
+  const int64_t n_groups = ((int64_t)n_lens + kGroup - 1) / kGroup;
   return trace_fixed_bytes(n_rb) + (size_t)trace_chunk_groups(n_rb, n_groups) * trace_group_bytes(n_rb);
 }
 
-cudaError_t launch_trace_split(const rsdev::FieldDev& f, double or0, double or1, double sp0, double sp1,
-                               const int64_t* ij, int64_t k, double* y, double* alpha, double* err, void* ws,
-                               cudaStream_t s) {
+// At most kTraceSplitRays rays.
+static void trace_split_block(const rsdev::FieldDev& f, double or0, double or1, double sp0, double sp1,
+                              const int64_t* ij, int64_t k, double* y, double* alpha, double* err, void* ws,
+                              cudaStream_t s) {
   const int64_t n_rb = (k + kRb - 1) / kRb, n_groups = ((int64_t)f.n_lens + kGroup - 1) / kGroup;
   const int64_t chunk = trace_chunk_groups(n_rb, n_groups);
   TraceWs w;
@@ -329,6 +331,15 @@ cudaError_t launch_trace_split(const rsdev::FieldDev& f, double or0, double or1,
                                                           g0 + chunk >= n_groups ? 1 : 0, w.xy, w.tmax, k, y, alpha,
                                                           err);
   }
+}
+
+cudaError_t launch_trace_split(const rsdev::FieldDev& f, double or0, double or1, double sp0, double sp1,
+                               const int64_t* ij, int64_t k, double* y, double* alpha, double* err, void* ws,
+                               cudaStream_t s) {
+  // blocks of rays, one after the other through the same workspace
+  for (int64_t r = 0; r < k; r += kTraceSplitRays)
+    trace_split_block(f, or0, or1, sp0, sp1, ij + 2 * r, std::min(kTraceSplitRays, k - r), y + 2 * r,
+                      alpha ? alpha + 2 * r : nullptr, err ? err + 2 * r : nullptr, ws, s);
   return cudaGetLastError();
 }
 

@@ -9,30 +9,34 @@ from gpu_helpers import rs
 
 pytestmark = pytest.mark.gpu
 
-DIRECT = 65537  # one ray more than the split path takes
+RAYS = 135000  # three blocks of the split path
 
 
 @pytest.mark.parametrize("mass", ["equal", "salpeter", "wide"])
-@pytest.mark.parametrize("n", [511, 512, 513, 575, 1023, 1280, 5001])
+@pytest.mark.parametrize("n", [511, 512, 513, 575, 640, 1023, 1280, 5001])
 def test_split_trace_equals_direct_trace(n, mass):
-    """Lens counts about group, renormalisation and tile boundaries; ray counts about a ray block, and (65536 rays,
-    5001 lenses) a workspace that takes the field in two chunks."""
+    """Lens counts about group, renormalisation and tile boundaries; ray counts about a ray block, a workspace that
+    takes the field in two chunks (65536 rays, 5001 lenses) and blocks of rays one after the other.  The direct
+    kernel runs where the workspace is refused."""
     m = rs()
     spec = ri.disc_field("tr", n, 0.5, 0.1, 0.3, 512, 64, seed=5, mass="equal" if mass == "equal" else "salpeter")
     masses = spec.masses if mass != "wide" else (spec.masses.astype(np.float64) * 2.0 ** 65).astype(np.float32)
-    ij = torch.from_numpy(ri.sample_rays(spec.grid, DIRECT, seed=n))
+    ij = torch.from_numpy(ri.sample_rays(spec.grid, RAYS, seed=n))
     f = m.Field(spec.lens_xy, masses, spec.kappa_c, spec.gamma)
     v = f.view(256, n - 256)  # the lens arrays of a view start inside its parent's
     try:
         for g in (f, v):
+            m.rs_set_alloc_failure(0)
             want = [t.cpu().numpy() for t in g.trace(spec.grid, ij, with_alpha=True, with_err=True)]
-            for k in (1, 127, 128, 129, 4000, 65536) if g is f else (300,):
+            m.rs_set_alloc_failure(-1)
+            for k in (1, 127, 128, 129, 511, 512, 4000, 65536, 65537, RAYS) if g is f else (300, 700):
                 got = [t.cpu().numpy() for t in g.trace(spec.grid, ij[:k], with_alpha=True, with_err=True)]
                 for a, b in zip(got, want):
                     assert np.array_equal(a, b[:k], equal_nan=True), k
             y = g.trace(spec.grid, ij[:200]).cpu().numpy()
             assert np.array_equal(y, want[0][:200], equal_nan=True)
     finally:
+        m.rs_set_alloc_failure(-1)
         v.close()
         f.close()
 
