@@ -241,7 +241,10 @@ int rs_set_staged_state_budget(uint64_t bytes);  /* also used by rs_shoot_stream
  * partition 0), and the last call (last = 1) bins them.  With the same partitions, the counts equal those
  * of rs_shoot_staged bit for bit.  Partitions as rs_shoot_staged (multiples of 256 lenses but the last;
  * masses given to all or to none); weighted = 1 runs every pass with per-lens masses (required when any
- * partition's masses are not all 1; every pass and re-evaluation of a shoot must use the same value).
+ * partition's masses are not all 1), weighted = 2 with masses weighed as in a field with a mass above 2^64
+ * (to be used when any partition has one: rs_shoot_staged then weighs all its partitions so, while at 1 only
+ * that partition is, and the float32 sums of the others differ by rounding).  Every pass and re-evaluation of a
+ * shoot must use the same value.
  *   rs_partition_buffer_bytes: device bytes of the state (28 per ray, padded to CTA tiles), of the list
  *     (16 + 8 per entry; capacity max(4096, rays/32)) and of d_ff (16 per entry) for the row block.
  * Calls are asynchronous on `stream`; buffers are caller-owned device memory.

@@ -402,7 +402,12 @@ def _byte_ptr(t, name, nbytes):
     return t.data_ptr()
 
 
-def rs_partition_pass(handle, weighted: bool, grid, row_begin: int, row_end: int, window, state, first: bool,
+def _weighted(weighted) -> int:
+    """0, 1 (also True), or 2: some partition of the shoot has a mass above 2^64."""
+    return 2 if weighted == 2 else int(bool(weighted))
+
+
+def rs_partition_pass(handle, weighted: int, grid, row_begin: int, row_end: int, window, state, first: bool,
                       last: bool, counts=None, out_of_window=None, lst=None, stream=None):
     """One lens partition's pass over rows [row_begin, row_end): adds its lenses to `state`; the last one maps
     and bins into counts / out_of_window and lists the rays to re-evaluate in `lst` (device byte buffers of
@@ -412,13 +417,13 @@ def rs_partition_pass(handle, weighted: bool, grid, row_begin: int, row_end: int
     pc = _dptr(counts, _COUNT_DTYPES, "counts", npx) if last else None
     po = _dptr(out_of_window, _OOW_DTYPES, "out_of_window", 1) if last else None
     g, w = _cgrid(grid), _cwin(window)
-    _check(load().rs_partition_pass(handle, int(bool(weighted)), ctypes.byref(g), int(row_begin), int(row_end),
+    _check(load().rs_partition_pass(handle, _weighted(weighted), ctypes.byref(g), int(row_begin), int(row_end),
                                     ctypes.byref(w), _byte_ptr(state, "state", sb), int(bool(first)), int(bool(last)),
                                     pc, po, _byte_ptr(lst, "list", lb) if last else None, _stream(stream)),
            "rs_partition_pass")
 
 
-def rs_partition_recheck(handle, weighted: bool, grid, row_begin: int, row_end: int, window, lst, ff, first: bool,
+def rs_partition_recheck(handle, weighted: int, grid, row_begin: int, row_end: int, window, lst, ff, first: bool,
                          last: bool, counts=None, out_of_window=None, stream=None):
     """One lens partition's float-float share of the listed rays (added to ff); the last call bins them."""
     _, lb, fb = rs_partition_buffer_bytes(grid, row_begin, row_end)
@@ -426,7 +431,7 @@ def rs_partition_recheck(handle, weighted: bool, grid, row_begin: int, row_end: 
     pc = _dptr(counts, _COUNT_DTYPES, "counts", npx) if last else None
     po = _dptr(out_of_window, _OOW_DTYPES, "out_of_window", 1) if last else None
     g, w = _cgrid(grid), _cwin(window)
-    _check(load().rs_partition_recheck(handle, int(bool(weighted)), ctypes.byref(g), int(row_begin), int(row_end),
+    _check(load().rs_partition_recheck(handle, _weighted(weighted), ctypes.byref(g), int(row_begin), int(row_end),
                                        ctypes.byref(w), _byte_ptr(lst, "list", lb), _byte_ptr(ff, "ff", fb),
                                        int(bool(first)), int(bool(last)), pc, po, _stream(stream)),
            "rs_partition_recheck")

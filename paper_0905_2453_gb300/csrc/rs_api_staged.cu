@@ -312,9 +312,10 @@ int partition_desc(rs_field_t part, int weighted, const rs_ray_grid* g, int64_t 
     return fail(RS_EINVAL, "the partition's masses are not all 1: every pass of the shoot must be weighted");
   if ((rc = check_field_device(part)) != RS_OK) return rc;
   if ((rc = fill_desc(part, g, row_begin, row_end, w, d_counts, d_oow, d)) != RS_OK) return rc;
-  // a partition above the kMass bound weighs its own lenses the wide way (the other partitions may be held by
-  // other processes, which do not see its masses: their kMass terms then differ from a single field's by rounding)
-  d->f.has_mass = weighted ? std::max<int>(rsdev::kMass, part->dev.has_mass) : rsdev::kUnitMass;
+  // the wide way (rsdev::kWideMass) where the caller says that some partition, perhaps of another process, has a
+  // mass above the kMass bound, and for a partition that has one itself whatever the caller says
+  const int mode = weighted == 2 ? rsdev::kWideMass : rsdev::kMass;
+  d->f.has_mass = weighted ? std::max<int>(mode, part->dev.has_mass) : rsdev::kUnitMass;
   return RS_OK;
 }
 

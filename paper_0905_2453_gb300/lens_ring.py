@@ -28,6 +28,15 @@ def ray_blocks(row_begin: int, row_end: int, block_rows: int) -> List[Tuple[int,
     return [(b, min(b + block_rows, row_end)) for b in range(row_begin, row_end, block_rows)]
 
 
+def partition_weight(masses) -> int:
+    """`weighted` that a partition of these masses (None or an array) needs: 0 where all are 1, 2 where one is above
+    2^64, else 1.  A shoot uses the largest of its partitions' values on every process."""
+    import numpy as np
+    if masses is None or len(masses) == 0 or bool(np.all(np.asarray(masses) == 1.0)):
+        return 0
+    return 2 if float(np.max(masses)) > 2.0 ** 64 else 1
+
+
 def rank_program(rank: int, world: int, blocks: Sequence[Tuple[int, int]], ops, certify: bool):
     """The schedule of one process of the ring (a generator yielding its transfers; see the module text).
 
@@ -103,12 +112,12 @@ class DeviceOps:
     ray blocks, and device buffers (two state buffers used by block parity; a list and a float-float buffer per
     block).  counts / out_of_window receive the map on the last process."""
 
-    def __init__(self, part, weighted: bool, grid, window, blocks, counts=None, out_of_window=None, stream=None,
+    def __init__(self, part, weighted: int, grid, window, blocks, counts=None, out_of_window=None, stream=None,
                  device=None):
         import torch
 
         from . import rs_partition_buffer_bytes
-        self.part, self.weighted, self.grid, self.window = part, bool(weighted), grid, window
+        self.part, self.weighted, self.grid, self.window = part, weighted, grid, window
         self.counts, self.out_of_window, self.stream = counts, out_of_window, stream
         dev = device if device is not None else torch.device("cuda", torch.cuda.current_device())
         sizes = [rs_partition_buffer_bytes(grid, b, e) for b, e in blocks]
@@ -137,12 +146,12 @@ class DeviceOps:
                              self._ff[k], first, last, self.counts, self.out_of_window, self.stream)
 
 
-def shoot_lens_ring(part, weighted: bool, grid, row_begin: int, row_end: int, window, counts, out_of_window,
+def shoot_lens_ring(part, weighted: int, grid, row_begin: int, row_end: int, window, counts, out_of_window,
                     rank: int, world: int, block_rows: int = 256, stream=None, group=None) -> None:
     """This process's share of a lens-partitioned shoot over rows [row_begin, row_end) with torch.distributed
     transfers between the holders of the partitions (process r holds partition r).  The counts accumulate on
-    the last process (world - 1); `weighted` must be the same everywhere (1 if any partition's masses are not
-    all 1)."""
+    the last process (world - 1); `weighted` must be the same everywhere: the largest ``partition_weight`` of the
+    partitions (1 if any one's masses are not all 1, 2 if any one has a mass above 2^64)."""
     from . import rs_get_certified_binning
     blocks = ray_blocks(row_begin, row_end, block_rows)
     ops = DeviceOps(part, weighted, grid, window, blocks, counts, out_of_window, stream)

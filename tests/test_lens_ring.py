@@ -192,3 +192,38 @@ def test_device_ring_two_partitions_equals_staged_shoot():
     finally:
         for p in parts:
             p.close()
+
+
+def test_partition_weight():
+    from paper_0905_2453_gb300.lens_ring import partition_weight
+    one = np.ones(4, np.float32)
+    assert [partition_weight(m) for m in (None, one[:0], one, 0.5 * one, 2.0 ** 64 * one)] == [0, 0, 0, 1, 1]
+    assert partition_weight(np.float32(2.0 ** 64 * (1 + 2.0 ** -23)) * one) == 2
+
+
+@pytest.mark.gpu
+def test_ordinary_partition_next_to_one_of_huge_masses():
+    """A partition's state under weighted = 2 is that of the same lenses inside a field with a mass above 2^64 (a view
+    of it takes its mode), bit for bit; under weighted = 1 it differs by rounding."""
+    from gpu_helpers import dev, rs
+    m = rs()
+    import rs_inputs as ri
+    spec = ri.disc_field("ring-wide", 600, 0.45, 0.05, 0.3, 200, 64, seed=8, mass="salpeter")
+    huge = spec.masses.copy()
+    huge[512:] *= np.float32(2.0 ** 70)
+    whole = m.Field(spec.lens_xy, huge, spec.kappa_c, spec.gamma)
+    part = m.Field(spec.lens_xy[:512], spec.masses[:512], spec.kappa_c, spec.gamma)
+    view = whole.view(0, 512)
+    try:
+        states = []
+        for f, weighted in ((view, 1), (part, 2), (part, 1)):
+            st = torch.zeros(m.rs_partition_buffer_bytes(spec.grid, 0, 200)[0], dtype=torch.uint8, device=dev())
+            m.rs_partition_pass(f.handle, weighted, spec.grid, 0, 200, spec.window, st, True, False)
+            torch.cuda.synchronize()
+            states.append(st)
+        assert torch.equal(states[0], states[1])
+        assert not torch.equal(states[0], states[2])
+    finally:
+        view.close()
+        whole.close()
+        part.close()
