@@ -434,7 +434,10 @@ typedef struct {
  * a guard band of the cut, so the set of pixels is that of a float64 evaluation.  Weights are
  * float32 (expf of the float32 exponent), sums are compensated float32 pairs; mu(y) carries a
  * relative error of a few 1e-7 (rows of the support are summed in float32, at most 2 R / pix + 3
- * terms each, then folded into compensated pairs).  The descriptor table is allocated stream-ordered
+ * terms each, then folded into compensated pairs).  In calls of few samples several threads share a
+ * sample's rows, so mu(y) may differ in rounding (some 1e-14) between calls with different numbers of
+ * samples, different largest supports or on devices of different size; a call repeated on a device
+ * gives the same bits.  The descriptor table is allocated stream-ordered
  * (cudaMallocAsync) and freed on the stream.
  * Errors: RS_EINVAL (argument), RS_EOVERFLOW (more than 2^40 samples), RS_ENOMEM, RS_ECUDA.
  */

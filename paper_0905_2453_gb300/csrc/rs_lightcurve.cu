@@ -284,6 +284,13 @@ void launch_lc(int parts, const LcTrack* tracks, int n_tracks, int64_t n_samples
 
 namespace rsint {
 
+// One, two, four and eight parts, us, the maps in L2, 152 SMs (one thread per sample as before: first figure):
+//   * few samples, wide supports: 18864 samples, discs of 34 rows 44 / 26 / 17 / 15, Gaussians of 48 rows 73 / 40 / 26 /
+//     21; 32000 samples, discs of 48 rows 81 / 49 / 41 / 36.  Narrow supports have nothing to share: 4000 samples, 6
+//     rows 10.8 / 8.5 / 7.6 / 6.4.
+//   * 4 x 256 threads per SM and more: dividing a sample costs more than idle SMs, 655360 samples, 14 rows
+//     60 / 74 / 99 / 126.  The wider the support the later that is (192000 samples, 48 rows 124 / 81 / 67 / 71; 655360
+//     samples, 34 rows 152 / 129 / 135 / 167): the one limit for all is on the safe side of the widest.
 int lc_parts(int sms, int64_t n_samples, double max_rows) {
   int parts = 1;
   while (parts < 8 && n_samples * parts < (int64_t)sms * 4 * kLcThreads && max_rows >= 8.0 * parts) parts *= 2;
