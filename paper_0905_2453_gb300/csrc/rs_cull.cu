@@ -16,7 +16,7 @@
 //
 // x4 zoom of the 1e4-lens map, 4.12e6 rays in the window: 8.52e6 rays shot with cells of 16 x 16 and no linear term
 // (|alpha(x) - alpha(c)| <= rho sum m / (d (d - rho))), 6.78e6 with it -- most of the rest in cells a few rho from a
-// lens, whose area shrinks with the cell's -- hence the cells of 8 x 8.
+// lens, whose area shrinks with the cell's -- hence the cells of 8 x 8: 5.08e6.
 #include <algorithm>
 
 #include "rs_internal.h"

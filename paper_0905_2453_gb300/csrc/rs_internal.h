@@ -135,7 +135,7 @@ cudaError_t launch_cull(const rsdev::ShootDesc& d, double hi0, double hi1, unsig
 cudaError_t launch_shoot_cells(const rsdev::ShootDesc& d, bool mid_cells, const unsigned* list, const unsigned* n_kept,
                                int grid, cudaStream_t s);
 
-// Lens-partitioned shooting (rs_staged.cu), default launch shape (4 warps x 8 rays): the per-ray
+// Lens-partitioned shooting (rs_staged.cu), one launch shape (4 warps x 8 rays, kTile lenses per stage): the per-ray
 // accumulator state of a call of n_rows x n0 rays takes staged_state_bytes; launch_staged adds the
 // partition d.f to it (first: start from zero; last: map and bin instead of storing).  The listed
 // rays of certified binning are re-evaluated partition by partition into ff (16 bytes per entry)

@@ -5,9 +5,10 @@
 // of (mostly) one track, so the warp's loads of neighbouring pixels fall in the same L1 lines and every per-sample
 // float64 step (position, box, quotient) is paid once per sample, not once per pixel.  A thread
 // walks the rows of the box that bounds its profile's support and, per row, the chord of the
-// support (a margin of ~2^-10 pixel each side).  With E = (di)^2 a0 + (dj)^2 a1 the float32 exponent of
-// the pixel offset (di, dj) in pixel units, the chord's interior (E below the cut by more than a
-// guard band, same margin) is summed without tests; at the rim membership is decided from
+// support.  On nearly every row no pixel centre lies within 2^-13 pixel (and the guard band below) of either end of
+// the chord, and the pixels between the ends are summed without tests.  On the others, with E = (di)^2 a0 + (dj)^2 a1
+// the float32 exponent of the pixel offset (di, dj) in pixel units, the chord's interior (E below the cut by more than
+// a guard band, a margin of ~2^-10 pixel) is summed without tests; at the rim membership is decided from
 // E, and pixels whose E lies within the guard band repeat the float64 test
 // ((lo + (i + 0.5) pix) - y)^2 + (...)^2 <= cut^2 (no fused multiply-add), so the covered pixel set
 // is exactly that of a float64 evaluation.

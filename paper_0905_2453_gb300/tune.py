@@ -42,8 +42,8 @@ def cache_key(field, grid) -> str:
 
 
 def wave_rows(n0: int, block: int, rpt: int, sms: int, ctas_per_sm: int = 2) -> int:
-    """The smallest number of grid rows whose CTAs (of `block` threads x `rpt` rays per thread, one warp per
-    row and 32 x rpt columns per CTA) fill whole waves of ctas_per_sm x sms CTAs (the default, two resident
+    """The smallest number of grid rows whose CTAs (of `block` threads x `rpt` rays per thread, as many rows as
+    warps and 32 x rpt columns per CTA) fill whole waves of ctas_per_sm x sms CTAs (the default, two resident
     CTAs per SM, makes whole waves at one or two)."""
     warps, seg = block // 32, 32 * rpt
     cpr = -(-int(n0) // seg)  # CTAs per group of `warps` rows
