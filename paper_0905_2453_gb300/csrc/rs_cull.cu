@@ -54,7 +54,7 @@ __device__ __forceinline__ void fold(float& hi, float& lo, float p) {
 // so that a level of few cells still fills the chip, and leave each thread 64 lenses or more (each has the float64
 // bound of its cell to work out as well).  With one thread per cell a level takes as long as one thread's walk over
 // all lenses, however few its cells are: 30000 lenses, 500^2 rays 1.17 ms for each of the three levels, call 5.58 ->
-// 2.56 ms; 64 lenses a thread against none at 60 lenses, 3600^2 rays 94 against 160 us.
+// 2.53 ms; 64 lenses a thread against none at 60 lenses, 3600^2 rays 94 against 160 us.
 __host__ __device__ __forceinline__ int cull_lanes(int64_t cells, int64_t threads, int n_lens) {
   int lanes = 1;
   while (lanes < 32 && cells * (2 * lanes) <= threads && n_lens >= 128 * lanes) lanes *= 2;
@@ -70,8 +70,10 @@ __device__ __forceinline__ double sum_over_lanes(double v, int lanes) {
 // the cell's source-plane box against the window.  Kept cells are appended to `out`; skipped cells add
 // their rays to the out-of-window count.  The first level takes every cell of the call (parent == nullptr), the
 // others the split x split cells of every kept cell of the level before.
+// Three CTAs per SM, 80 registers: at the four that the compiler aims at the lens loop spills (x4 zoom of 1e4 lenses, a
+// lower level: 1.17 ms, 0.85 so).
 template <bool MASS>
-__global__ void __launch_bounds__(kCullBlock)
+__global__ void __launch_bounds__(kCullBlock, 3)
     cull_kernel(const ShootDesc d, int cell_rays, int64_t n_cx, int64_t n_cells, const unsigned* __restrict__ parent,
                 const unsigned* __restrict__ parent_count, int64_t n_px, int split, int64_t threads, double hi0,
                 double hi1, unsigned* __restrict__ out, unsigned* __restrict__ out_count, unsigned long long* __restrict__ n_shot) {
@@ -111,20 +113,14 @@ __global__ void __launch_bounds__(kCullBlock)
   float q1h = 0.f, q1l = 0.f, q2h = 0.f, q2l = 0.f;
   bool near = false;
   const int n = d.f.n_lens;
-  float4 next = make_float4(0.f, 0.f, 0.f, 0.f);  // the thread's lens of the tile after the one summed
-  float next_m = 0.f;
-  auto fetch = [&](int l) {
-    if (l >= n) return;
-    next = d.f.lens4[l];
-    if (MASS) next_m = d.f.mass2[l].x;
-  };
-  fetch((int)threadIdx.x);
   for (int t0 = 0; t0 < n; t0 += kCullBlock) {
     __syncthreads();
-    s_lens[threadIdx.x] = next;
-    if (MASS) s_mass[threadIdx.x] = next_m;
+    const int l = t0 + threadIdx.x;
+    if (l < n) {
+      s_lens[threadIdx.x] = d.f.lens4[l];
+      if (MASS) s_mass[threadIdx.x] = d.f.mass2[l].x;
+    }
     __syncthreads();
-    if (n - t0 > kCullBlock) fetch(t0 + kCullBlock + (int)threadIdx.x);
     const int cnt = min(kCullBlock, n - t0);
     for (int g = 0; g < cnt; g += 32 * lanes) {  // at most 32 terms of the thread
       float pa1 = 0.f, pa2 = 0.f, pb = 0.f, ps = 0.f, pq1 = 0.f, pq2 = 0.f;
