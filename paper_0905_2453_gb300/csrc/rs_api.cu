@@ -861,6 +861,7 @@ int rs_shoot_culled(rs_field_t f, const rs_ray_grid* g, int64_t row_begin, int64
   if (saves) {
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     mid_cells = cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone;
+    (void)cudaGetLastError();
   }
   void* ws = nullptr;
   cudaError_t e = dev_alloc_async(&ws, mid_cells ? list_off : full, s);
