@@ -181,9 +181,9 @@ int rs_shoot_rows(rs_field_t f, const rs_ray_grid* g, int64_t row_begin, int64_t
  * shot cells use the same per-ray arithmetic and binning, certified binning included).
  *   d_rays_shot : uint64 device counter or NULL; ACCUMULATES the number of rays actually shot.
  * Other arguments, accumulation and errors as rs_shoot_rows.  Workspace is allocated
- * stream-ordered (4 bytes per cell plus the re-evaluation list).  Where that much cannot be had, and
- * while the stream is being captured, calls of more than 2 MiB of cells shoot cells of 16 x 16, with a
- * quarter of it: more rays, the same results.
+ * stream-ordered (4 bytes per cell plus the re-evaluation list).  Fields of less than 256 lenses, and calls of
+ * more than 2 MiB of cells where that much cannot be had or while the stream is being captured, shoot
+ * cells of 16 x 16, with a quarter of it: more rays, the same results.
  */
 int rs_shoot_culled(rs_field_t f, const rs_ray_grid* g, int64_t row_begin, int64_t row_end, const rs_window* w,
                     uint32_t* d_counts, uint64_t* d_out_of_window, uint64_t* d_rays_shot, void* stream);
